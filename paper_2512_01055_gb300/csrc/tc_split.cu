@@ -55,7 +55,7 @@
 //
 // Warp roles of the W-term kernel (384 threads): warps 0, 10 and 11 issue the
 // bulk copies (a warp completes about one stage per ~0.37 us, several warps
-// overlap), warp 1 owns TMEM and lane 0 issues the MMAs, warps 2-9 drain TMEM
+// overlap), warp 1 owns TMEM and its elected lane issues the MMAs, warps 2-9 drain TMEM
 // (warp w reads TMEM lanes 32 (w % 4) .. +31, half the columns each).
 // Every mbarrier wait is bounded; on expiry the kernel records an error code,
 // lets every role leave its loop, waits (bounded) for its own copies and MMAs
@@ -303,69 +303,87 @@ tc_wterm_kernel(const __grid_constant__ WtBatch B) {
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int stage = 0, jc = 0;
-      uint32_t phase = 0, aphase = 0;
-      bool ok = true;
-      for (long long gi = blockIdx.x; ok && gi < B.total_items; gi += gridDim.x) {
-        while (jc + 1 < B.njobs && gi >= B.job[jc + 1].item0) ++jc;
-        const WtJob &J = B.job[jc];
-        const int nc = J.g.nc;
-        const int nkb = J.g.hv + J.g.ho;
-        const int nchain = (nkb + KCHAIN - 1) / KCHAIN;
-        const uint32_t id = idesc(128, nc);
-        const uint32_t ahb = (uint32_t)S * A_HALF, bhb = (uint32_t)S * nc * 16;
-        for (int ch = 0; ok && ch < nchain; ++ch) {
-          const int kc0 = ch * nkb / nchain, kc1 = (ch + 1) * nkb / nchain;
-          // A new item needs both accumulators back from the drain.  A later
-          // chain needs only L0, which the drain is still reading: its first
-          // ndef K blocks issue their L1 products first, and their level-0
-          // products (in K order, the first one restarting L0) follow once L0
-          // is free, so the tensor pipe keeps working meanwhile.
-          if (ch == 0) {
-            if (!mbar_wait(&accempty_bar, aphase ^ 1u, &abort_flag, B.err, ERR_TIMEOUT_ACCEMPTY)) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          }
-          const int ndef = ch > 0 ? min(DEFER, kc1 - kc0) : 0;
-          int dstage[DEFER];
-          for (int kc = kc0; kc < kc1; ++kc) {
-            if (!mbar_wait(&full_bar[stage], phase, &abort_flag, B.err, ERR_TIMEOUT_FULL)) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t sA = smem_u32(sm + (size_t)stage * B.slot);
-            const uint32_t sB = sA + 2 * ahb;
+    // The whole warp walks the K blocks, so stages, descriptors and phases stay
+    // warp-uniform, and one elected lane issues.  With the loop under
+    // `lane == 0` instead the issue itself was the limit: an MMA of M = 128,
+    // K = 16 took 56 ns whatever its width below N = 208 and 62 ns with the
+    // operand copies running; issued this way it takes 40 ns up to N = 160 and
+    // 53.5 ns (the tensor pipe's rate) at N = 208, with and without copies
+    // (2.0 GHz, six slice pairs per K block).
+    const uint32_t el = elect_one();
+    const uint32_t sbase = smem_u32(sm), slot = (uint32_t)B.slot;
+    int stage = 0, jc = 0;
+    uint32_t phase = 0, aphase = 0;
+    bool ok = true;
+    for (long long gi = blockIdx.x; ok && gi < B.total_items; gi += gridDim.x) {
+      while (jc + 1 < B.njobs && gi >= B.job[jc + 1].item0) ++jc;
+      const WtJob &J = B.job[jc];
+      const uint32_t nc = (uint32_t)J.g.nc;
+      const int nkb = J.g.hv + J.g.ho;
+      const int nchain = (nkb + KCHAIN - 1) / KCHAIN;
+      const uint32_t id = idesc(128, (int)nc);
+      const uint32_t ahb = (uint32_t)S * A_HALF, bhb = (uint32_t)S * nc * 16;
+      // descriptors of slice 0 at stage address 0: adding (address >> 4) moves them
+      const uint64_t da0 = sdesc(0, ahb), db0 = sdesc(0, bhb) + ((2 * ahb) >> 4);
+      for (int ch = 0; ok && ch < nchain; ++ch) {
+        const int kc0 = ch * nkb / nchain, kc1 = (ch + 1) * nkb / nchain;
+        // A new item needs both accumulators back from the drain.  A later
+        // chain needs only L0, which the drain is still reading: its first
+        // ndef K blocks issue their L1 products first, and their level-0
+        // products (in K order, the first one restarting L0) follow once L0
+        // is free, so the tensor pipe keeps working meanwhile.
+        if (ch == 0) {
+          if (!mbar_wait(&accempty_bar, aphase ^ 1u, &abort_flag, B.err, ERR_TIMEOUT_ACCEMPTY)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        const int ndef = ch > 0 ? min(DEFER, kc1 - kc0) : 0;
+        const int stage0 = stage;                                                  // the chain's first stage
+        for (int kc = kc0; kc < kc1; ++kc) {
+          if (!mbar_try(smem_u32(&full_bar[stage]), phase) &&
+              !mbar_wait(&full_bar[stage], phase, &abort_flag, B.err, ERR_TIMEOUT_FULL)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t at = (sbase + (uint32_t)stage * slot) >> 4;
+          const uint64_t da = da0 + at, db = db0 + at;
+          const bool deferred = kc - kc0 < ndef;
+          if (el) {
             int n = 0;
 #pragma unroll
             for (int a = 0; a < S; ++a)
 #pragma unroll
               for (int b = 0; b < S - a; ++b) {
                 if (a + b == 0) continue;                                          // levels >= 1 -> L1
-                mma_bf16(tbase + (uint32_t)nc, sdesc(sA + a * A_HALF, ahb), sdesc(sB + b * nc * 16, bhb), id,
+                mma_bf16(tbase + nc, da + (uint32_t)(a * (A_HALF >> 4)), db + (uint32_t)b * nc, id,
                          (kc == 0 && n == 0) ? 0u : 1u);
                 ++n;
               }
-            if (kc - kc0 < ndef) {
-              dstage[kc - kc0] = stage;                                            // level 0 deferred
-              if (++stage == B.stages) { stage = 0; phase ^= 1u; }
-              if (kc - kc0 + 1 < ndef) continue;
-              if (!mbar_wait(&accempty_bar, aphase ^ 1u, &abort_flag, B.err, ERR_TIMEOUT_ACCEMPTY)) { ok = false; break; }
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              for (int d = 0; d < ndef; ++d) {
-                const uint32_t dA = smem_u32(sm + (size_t)dstage[d] * B.slot), dB = dA + 2 * ahb;
-                mma_bf16(tbase, sdesc(dA, ahb), sdesc(dB, bhb), id, d > 0 ? 1u : 0u);   // level 0 -> L0
-                mma_commit(&empty_bar[dstage[d]]);
-              }
-              continue;
+            if (!deferred) {
+              mma_bf16(tbase, da, db, id, kc > kc0 ? 1u : 0u);                     // level 0 -> L0
+              mma_commit(&empty_bar[stage]);
             }
-            mma_bf16(tbase, sdesc(sA, ahb), sdesc(sB, bhb), id, kc > kc0 ? 1u : 0u);  // level 0 -> L0
-            mma_commit(&empty_bar[stage]);
-            if (++stage == B.stages) { stage = 0; phase ^= 1u; }
           }
-          if (!ok) break;
-          mma_commit(&accfull_bar);
-          aphase ^= 1u;
+          if (++stage == B.stages) { stage = 0; phase ^= 1u; }
+          if (deferred && kc - kc0 + 1 == ndef) {
+            // the deferred level-0 products, from the chain's first ndef stages
+            if (!mbar_wait(&accempty_bar, aphase ^ 1u, &abort_flag, B.err, ERR_TIMEOUT_ACCEMPTY)) { ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            int ds = stage0;
+            for (int d = 0; d < ndef; ++d) {
+              const uint32_t dat = (sbase + (uint32_t)ds * slot) >> 4;
+              if (el) {
+                mma_bf16(tbase, da0 + dat, db0 + dat, id, d > 0 ? 1u : 0u);        // level 0 -> L0
+                mma_commit(&empty_bar[ds]);
+              }
+              if (++ds == B.stages) ds = 0;
+            }
+          }
         }
+        if (!ok) break;
+        if (el) mma_commit(&accfull_bar);
+        aphase ^= 1u;
       }
-      // all MMAs issued by this thread complete before TMEM is released
+    }
+    if (el) {
+      // all MMAs issued by this lane complete before TMEM is released
       mma_commit(&teardown_bar);
       const uint32_t a = smem_u32(&teardown_bar);
       for (long long it = 0; it < WAIT_LIMIT && !mbar_try(a, 0); ++it) {
