@@ -103,7 +103,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   double *dout = (double *)(base + L.out);
   TC_CUDA(ctx, cudaMemsetAsync(w.counter, 0, 2 * sizeof(unsigned), st));
   if (e_ijk_dev) TC_CUDA(ctx, cudaMemsetAsync(e_ijk_dev, 0, sizeof(double) * (size_t)o * o * o, st));
-  int launches = 1;                                      // reduce_jobs
+  int launches = d.n_trip > 0 ? 2 : 1;                   // the reduction
   int nblocks = 0;                                       // split path: blocks of triplets
   if (stg && (!split || subset)) return fail(ctx, TC_EINTERNAL, "staged inputs need the split path on all triplets");
   int staged = 0;                                        // chunks sliced so far

@@ -188,7 +188,7 @@ int *df_error_flag(void *scratch, int o, int v, int nq);
 struct RedJob {
   int n_trip, items_per_trip, o;
   const int4 *trip;
-  const double *partial;
+  double *partial;       // [n_trip][items_per_trip][2]; each triplet's first pair is overwritten by its sums
   double *e_trip;        // [n_trip] weighted triplet contributions
   double *e_ijk;         // optional [o][o][o]
   double *out;           // [3]: E, sum |e| and E[5]_ST
