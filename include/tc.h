@@ -57,7 +57,12 @@ typedef enum {
 } tc_status;
 
 typedef enum {
-  TC_FP64 = 0,         /* W built with FP64 tensor-core (DMMA) tiles, FP64 everywhere */
+  TC_FP64 = 0,         /* FP64-accurate W, FP64 epilogue and sums.  W as exact integer products in residues on
+                          the BF16 tensor cores: operands rounded once to a common power-of-two grid at least 2^-53
+                          of their norms, W to 64 bits (an error below that of FP64 accumulation); or with FP64
+                          tensor-core (DMMA) tiles where the shape (o < 2, v < 8, K = 2v + 2o padded above 1024),
+                          the memory (the residue images take at most a quarter of the budget) or the inputs
+                          (infinities, NaN, norms outside 2^+-100) do not allow it */
   TC_SPLIT_BF16 = 1    /* W built from BF16 slices on tcgen05 tensor cores, FP32 accumulation;
                           V and the Eq. 1 bracket in FP32; D, 1/D, each point's quotient and
                           the sums over a work item in float pairs (~48 significant bits);
@@ -90,13 +95,13 @@ typedef struct {
   int o, v;
   double queue_seconds;      /* serving: time from tc_submit to the start of its GPU work */
   double kernel_seconds;     /* device time of the W/V/energy kernels (CUDA events on the call's stream):
-                                FP64, the fused kernel; split path, all W-term and energy launches */
-  double prep_seconds;       /* device time of the slicing / re-layout kernels (split path), else 0 */
+                                all W and energy launches (FP64 by DMMA: the fused kernel) */
+  double prep_seconds;       /* device time of the slicing / residue / re-layout kernels, 0 for FP64 by DMMA */
   long long n_items;         /* energy work items (triplet x tile-orbit chunk) processed */
   int launches;              /* kernels this call launched */
   int reserved;
-  double wterm_seconds;      /* device time of the kernels that form W: FP64, the fused kernel (= kernel_seconds);
-                                split path, the W-term GEMM launches alone (blocking entry points only) */
+  double wterm_seconds;      /* device time of the kernels that form W: the GEMM launches alone (blocking entry
+                                points only); FP64 by DMMA, the fused kernel (= kernel_seconds) */
   double e_t5;               /* E[5]_ST: the part of E_(T) from the V factor of Eq. 1, sum (V r3(W))/D with the
                                 same weights; E[4] = e_t - e_t5 is the W r3(W)/D part (r3 is the bracket of Eq. 1) */
   double df_seconds;         /* tc_energy_df(_dev): device time of the integral assembly from the DF
@@ -120,7 +125,10 @@ tc_status tc_init(tc_ctx **ctx, const tc_options *opt);
  * kernel_seconds includes the later chunks' slicing and any wait for their
  * copies.  No copy reads the caller's arrays after the call returns.
  * prec: tc_precision, or < 0 for the context default.  slices: 2..4 for
- * TC_SPLIT_BF16, <= 0 for the default; ignored for TC_FP64.
+ * TC_SPLIT_BF16, <= 0 for the default; ignored for TC_FP64.  TC_FP64 holds
+ * residue images of the operands (30 bytes per element of ovvv in each of two
+ * orders) besides tc_workspace_bytes while the context's budget and the device
+ * have room for them; they are given back when another call needs the memory.
  * e_ijk (optional, may be NULL): host array [o][o][o] that receives the
  * weighted contribution of each occupied triplet i >= j >= k at [i][j][k]
  * (E_(T) is their sum); entries with i < j or j < k are set to 0. */
@@ -231,7 +239,8 @@ tc_status tc_combine_parts(const double *parts, int n, double *e_t);
  * streams while others compute.  Computation proceeds in iterations of about
  * iteration_ms: each iteration is one persistent multi-job launch (replayed
  * from a CUDA graph) over a slice of the items of every ready job of one
- * precision group, the slices shared fairly, so a job submitted while others
+ * precision group (a small batch first waits for a small job of its group that
+ * is being handed in or prepared), the slices shared fairly, so a job submitted while others
  * run starts within an iteration and small jobs are not stuck behind large
  * ones.  A job's result does not depend on the other jobs it ran with.
  * ------------------------------------------------------------------------ */
@@ -322,7 +331,8 @@ tc_status tc_energy_dev_noalloc(int o, int v, const double *eps, const double *t
                                 double *e_ijk_dev, void *stream, char *errbuf, size_t errlen);
 
 /* Device bytes a job of this shape and precision needs besides its inputs
- * (work tables, partial sums; split path also the BF16 operand images, FP32
+ * (work tables, partial sums; not the residue images TC_FP64 holds where there
+ * is room; split path also the BF16 operand images, FP32
  * copies and the W buffer of one block of triplets).  Pure host arithmetic. */
 size_t tc_workspace_bytes(int o, int v, int prec, int slices);
 

@@ -75,11 +75,12 @@ struct Staging {
 
 // The hot path on device-resident inputs.  Caller holds ctx->mu.
 // subset (optional): process these triplets only; e_sub receives their sums.
+// dmma (FP64): use the DMMA kernel whatever the shape.
 // stg (optional, split path, no subset): slice each chunk of the inputs once
 // it has arrived, just before the first block of triplets that reads it.
 tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, int slices, double *e_ijk_dev,
                      cudaStream_t st, tc_result *out, const std::vector<int4> *subset = nullptr,
-                     std::vector<double> *e_sub = nullptr, const Staging *stg = nullptr) {
+                     std::vector<double> *e_sub = nullptr, const Staging *stg = nullptr, bool dmma = false) {
   const bool split = (prec == TC_SPLIT_BF16);
   const int nt = split ? tc::split_tile() : tc::fp64_tile();
   const tc::Dims d = tc::plan::make_dims(o, v, nt, subset ? (int)subset->size() : -1,
@@ -88,8 +89,23 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   const tc::SplitLayout SL = split ? tc::split_layout(o, v, slices) : tc::SplitLayout{};
   const size_t need = L.total + SL.total;
   if (need > ctx->budget) return fail(ctx, TC_ENOMEM, "workspace %zu B exceeds budget %zu B", need, ctx->budget);
-  TC_CUDA(ctx, ctx->ws.ensure(L.total));
-  if (split) TC_CUDA(ctx, ctx->ws_split.ensure(SL.total));
+  TC_CUDA(ctx, ctx->grow(ctx->ws, L.total));
+  if (split) TC_CUDA(ctx, ctx->grow(ctx->ws_split, SL.total));
+  // FP64: on the tensor cores where the path covers the shape, its workspace
+  // takes at most a quarter of the budget (the rest stays for the caller's own
+  // arrays) and the device has the room; else the DMMA kernel.
+  const tc::RnsLayout RL = split ? tc::RnsLayout{} : tc::rns_layout(o, v, d.n_trip);
+  bool rns = !split && !dmma && d.n_trip > 0 && tc::rns_supported(o, v) && RL.total <= ctx->budget / 4 &&
+             need + RL.total + ctx->in_ovvv.cap + ctx->in_t2.cap + ctx->in_ovov.cap + ctx->in_ovoo.cap <= ctx->budget;
+  if (rns) {
+    const cudaError_t e = ctx->ws_rns.ensure(RL.total);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      rns = false;
+    } else {
+      TC_CUDA(ctx, e);
+    }
+  }
   char *base = (char *)ctx->ws.p;
   const std::vector<int4> tab = tc::plan::tables(d, L, subset);
   TC_CUDA(ctx, cudaMemcpyAsync(base + L.trip, tab.data(), tab.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
@@ -101,7 +117,8 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   w.err = (int *)(base + L.counter + sizeof(unsigned));
   double *e_trip = (double *)(base + L.e_trip);
   double *dout = (double *)(base + L.out);
-  TC_CUDA(ctx, cudaMemsetAsync(w.counter, 0, 2 * sizeof(unsigned), st));
+  TC_CUDA(ctx, cudaMemsetAsync(w.counter, 0, 3 * sizeof(unsigned), st));
+  tc::RnsTables rt;
   if (e_ijk_dev) TC_CUDA(ctx, cudaMemsetAsync(e_ijk_dev, 0, sizeof(double) * (size_t)o * o * o, st));
   int launches = d.n_trip > 0 ? 2 : 1;                   // the reduction
   int nblocks = 0;                                       // split path: blocks of triplets
@@ -135,19 +152,27 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
     TC_CUDA(ctx, tc::launch_split_prep(SL, in, ctx->ws_split.p, st));
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
     launches += tc::split_prep_launches();
+  } else if (rns) {
+    rt = tc::rns_tables(o, tab.data(), d.n_trip);
+    TC_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
+    TC_CUDA(ctx, tc::launch_rns_prep(RL, in, ctx->ws_rns.p, rt, subset == nullptr, w.err + 1, st));
+    TC_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
+    launches += tc::rns_prep_launches();
   }
   if (d.n_items > 0) {
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[0], st));
-    if (split) {
-      // blocks of nb triplets: the three W-term GEMM launches sum W into the
-      // W buffer, then the energy launch runs over the block's orbits
-      const int nb = SL.g.nb;
-      nblocks = (d.n_trip + nb - 1) / nb;
+    if (split || rns) {
+      nblocks = (d.n_trip + (split ? SL.g.nb : RL.g.nb) - 1) / (split ? SL.g.nb : RL.g.nb);
       while ((int)ctx->wev.size() < 2 * nblocks) {
         cudaEvent_t e = nullptr;
         TC_CUDA(ctx, cudaEventCreate(&e));
         ctx->wev.push_back(e);
       }
+    }
+    if (split) {
+      // blocks of nb triplets: the three W-term GEMM launches sum W into the
+      // W buffer, then the energy launch runs over the block's orbits
+      const int nb = SL.g.nb;
       static thread_local tc::WtBatch wb;
       static thread_local tc::EnBatch eb;
       for (int blk = 0; blk < nblocks; ++blk) {
@@ -167,6 +192,20 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
         TC_CUDA(ctx, tc::launch_split_block(wb, eb, slices, ctx->num_sms, st, ctx->wev[2 * blk], ctx->wev[2 * blk + 1]));
       }
       launches += (tc::SPLIT_WT_LAUNCHES + 1) * nblocks - 1;
+    } else if (rns) {
+      // blocks of nb triplets: the storing and the adding GEMM launch, then
+      // the energy launch over the block's orbits
+      static thread_local tc::RnBatch gb[tc::RNS_GEMM_LAUNCHES];
+      static thread_local tc::RnEnBatch eb;
+      const int nb = RL.g.nb;
+      for (int blk = 0; blk < nblocks; ++blk) {
+        const int t0 = blk * nb, nt = std::min(nb, d.n_trip - t0);
+        gb[0].njobs = gb[1].njobs = eb.njobs = 1;
+        gb[0].err = gb[1].err = w.err;
+        tc::rns_block(RL, ctx->ws_rns.p, d, in, w, rt, t0, nt, &gb[0].job[0], &gb[1].job[0], &eb.job[0]);
+        TC_CUDA(ctx, tc::launch_rns_block(gb, eb, ctx->num_sms, st, ctx->wev[2 * blk], ctx->wev[2 * blk + 1]));
+      }
+      launches += (tc::RNS_GEMM_LAUNCHES + 1) * nblocks - 1;
     } else {
       int per_sm = 0;
       TC_CUDA(ctx, tc::fp64_blocks_per_sm(&per_sm));
@@ -195,13 +234,16 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
     TC_CUDA(ctx, tc::launch_reduce(rb, st));
   }
   TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out, dout, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-  TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out + 3, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out + 3, w.err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   TC_CUDA(ctx, cudaStreamSynchronize(st));
-  int errflag = 0;
-  std::memcpy(&errflag, ctx->host_out + 3, sizeof(int));
+  int errs[2] = {0, 0};
+  std::memcpy(errs, ctx->host_out + 3, sizeof errs);
+  const int errflag = errs[0];
   if (errflag != 0)
     return fail(ctx, (errflag >= 11 && errflag <= 15) ? TC_ETIMEOUT : TC_EINTERNAL,
                 "device-side wait gave up (code %d)", errflag);
+  // inputs beyond the integer grid's range (infinities, NaN, norms outside 2^+-100): the DMMA kernel
+  if (rns && errs[1] != 0) return run_device(ctx, o, v, in, prec, slices, e_ijk_dev, st, out, subset, e_sub, stg, true);
   out->e_t = ctx->host_out[0];
   out->e_t5 = ctx->host_out[2];
   if (e_sub) {
@@ -216,7 +258,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
     TC_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]));
     out->kernel_seconds = 1e-3 * ms;
     out->wterm_seconds = out->kernel_seconds;
-    if (split) {
+    if (split || rns) {
       double wsum = 0.0;
       for (int blk = 0; blk < nblocks; ++blk) {
         TC_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->wev[2 * blk], ctx->wev[2 * blk + 1]));
@@ -233,7 +275,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
       psum += 1e-3 * ms;
     }
     out->prep_seconds = psum;
-  } else if (split) {
+  } else if (split || rns) {
     float ms = 0.f;
     TC_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev[2], ctx->ev[3]));
     out->prep_seconds = 1e-3 * ms;
@@ -260,10 +302,10 @@ size_t df_bytes(int o, int v, int nq) {
 tc_status df_energy(tc_ctx *ctx, int o, int v, int nq, const double *eps, const double *t1, const double *t2,
                     const double *B, int prec, int slices, double *e_ijk_dev, cudaStream_t st, tc_result *out) {
   const size_t n_ovvv = (size_t)o * v * v * v, n_ovoo = (size_t)o * v * o * o, n_ovov = (size_t)o * v * o * v;
-  TC_CUDA(ctx, ctx->in_ovvv.ensure(sizeof(double) * n_ovvv));
-  TC_CUDA(ctx, ctx->in_ovoo.ensure(sizeof(double) * n_ovoo));
-  TC_CUDA(ctx, ctx->in_ovov.ensure(sizeof(double) * n_ovov));
-  TC_CUDA(ctx, ctx->df_b.ensure(tc::df_scratch_bytes(o, v, nq)));
+  TC_CUDA(ctx, ctx->grow(ctx->in_ovvv, sizeof(double) * n_ovvv));
+  TC_CUDA(ctx, ctx->grow(ctx->in_ovoo, sizeof(double) * n_ovoo));
+  TC_CUDA(ctx, ctx->grow(ctx->in_ovov, sizeof(double) * n_ovov));
+  TC_CUDA(ctx, ctx->grow(ctx->df_b, tc::df_scratch_bytes(o, v, nq)));
   for (auto &e : ctx->dfev)
     if (!e) TC_CUDA(ctx, cudaEventCreate(&e));
   double *ovvv = (double *)ctx->in_ovvv.p, *ovoo = (double *)ctx->in_ovoo.p, *ovov = (double *)ctx->in_ovov.p;
@@ -361,6 +403,7 @@ void tc_finalize(tc_ctx *ctx) {
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   ctx->ws.release();
   ctx->ws_split.release();
+  ctx->ws_rns.release();
   ctx->in_eps.release(); ctx->in_t1.release(); ctx->in_t2.release();
   ctx->in_ovvv.release(); ctx->in_ovoo.release(); ctx->in_ovov.release();
   ctx->df_b.release();
@@ -438,10 +481,10 @@ tc_status tc_energy_df(tc_ctx *ctx, int o, int v, int nq, const double *eps, con
   const size_t need = in_bytes + df_bytes(o, v, nq) + tc_workspace_bytes(o, v, prec, slices);
   if (need > ctx->budget) return fail(ctx, TC_ENOMEM, "job needs %zu B, budget %zu B", need, ctx->budget);
   cudaStream_t st = ctx->stream;
-  TC_CUDA(ctx, ctx->in_eps.ensure(sizeof(double) * (n_eps + (size_t)o * o * o)));
-  TC_CUDA(ctx, ctx->in_t1.ensure(sizeof(double) * n_t1));
-  TC_CUDA(ctx, ctx->in_t2.ensure(sizeof(double) * n_t2));
-  TC_CUDA(ctx, ctx->df_in.ensure(sizeof(double) * n_b));
+  TC_CUDA(ctx, ctx->grow(ctx->in_eps, sizeof(double) * (n_eps + (size_t)o * o * o)));
+  TC_CUDA(ctx, ctx->grow(ctx->in_t1, sizeof(double) * n_t1));
+  TC_CUDA(ctx, ctx->grow(ctx->in_t2, sizeof(double) * n_t2));
+  TC_CUDA(ctx, ctx->grow(ctx->df_in, sizeof(double) * n_b));
   TC_CUDA(ctx, cudaMemcpyAsync(ctx->in_eps.p, eps, sizeof(double) * n_eps, cudaMemcpyHostToDevice, st));
   TC_CUDA(ctx, cudaMemcpyAsync(ctx->in_t1.p, t1, sizeof(double) * n_t1, cudaMemcpyHostToDevice, st));
   TC_CUDA(ctx, cudaMemcpyAsync(ctx->in_t2.p, t2, sizeof(double) * n_t2, cudaMemcpyHostToDevice, st));
@@ -586,12 +629,12 @@ tc_status tc_energy(tc_ctx *ctx, int o, int v, const double *eps, const double *
     return fail(ctx, TC_ENOMEM, "job needs %zu B, budget %zu B", in_bytes + tc_workspace_bytes(o, v, prec, slices),
                 ctx->budget);
   cudaStream_t st = ctx->stream;
-  TC_CUDA(ctx, ctx->in_eps.ensure(sizeof(double) * (n_eps + (size_t)o * o * o)));
-  TC_CUDA(ctx, ctx->in_t1.ensure(sizeof(double) * n_t1));
-  TC_CUDA(ctx, ctx->in_t2.ensure(sizeof(double) * n_t2));
-  TC_CUDA(ctx, ctx->in_ovvv.ensure(sizeof(double) * n_ovvv));
-  TC_CUDA(ctx, ctx->in_ovoo.ensure(sizeof(double) * n_ovoo));
-  TC_CUDA(ctx, ctx->in_ovov.ensure(sizeof(double) * n_ovov));
+  TC_CUDA(ctx, ctx->grow(ctx->in_eps, sizeof(double) * (n_eps + (size_t)o * o * o)));
+  TC_CUDA(ctx, ctx->grow(ctx->in_t1, sizeof(double) * n_t1));
+  TC_CUDA(ctx, ctx->grow(ctx->in_t2, sizeof(double) * n_t2));
+  TC_CUDA(ctx, ctx->grow(ctx->in_ovvv, sizeof(double) * n_ovvv));
+  TC_CUDA(ctx, ctx->grow(ctx->in_ovoo, sizeof(double) * n_ovoo));
+  TC_CUDA(ctx, ctx->grow(ctx->in_ovov, sizeof(double) * n_ovov));
   TC_CUDA(ctx, cudaMemcpyAsync(ctx->in_eps.p, eps, sizeof(double) * n_eps, cudaMemcpyHostToDevice, st));
   TC_CUDA(ctx, cudaMemcpyAsync(ctx->in_t1.p, t1, sizeof(double) * n_t1, cudaMemcpyHostToDevice, st));
   tc::Inputs in{(const double *)ctx->in_eps.p, (const double *)ctx->in_t1.p, (const double *)ctx->in_t2.p,

@@ -45,6 +45,7 @@ struct tc_ctx {
   cudaStream_t stream = nullptr;
   tc::DevBuf ws;                            // tables, partials and sums, reused across calls
   tc::DevBuf ws_split;                      // BF16 operand images, FP32 copies, W buffer
+  tc::DevBuf ws_rns;                        // FP64 tensor-core path: residue images, W buffer (given back when another buffer needs the room)
   tc::DevBuf in_eps, in_t1, in_t2, in_ovvv, in_ovoo, in_ovov;   // tc_energy's device copies; tc_energy_df_dev's integrals
   tc::DevBuf df_b;                          // tc_energy_df(_dev): scratch of the integral assembly (scales, digit images)
   tc::DevBuf df_in;                         // tc_energy_df: the device copy of B
@@ -55,6 +56,16 @@ struct tc_ctx {
   cudaStream_t copy_stream = nullptr;       // tc_energy: host-to-device copies of the inputs, by occupied-index chunk
   std::vector<cudaEvent_t> cev;             // tc_energy: one per chunk, recorded on copy_stream after its copies
   std::vector<cudaEvent_t> pev;             // staged split path: a pair around each chunk's slicing
+  // Grow a buffer; when the device is out of memory, the residue images give way.
+  cudaError_t grow(tc::DevBuf &b, size_t bytes) {
+    cudaError_t e = b.ensure(bytes);
+    if (e == cudaErrorMemoryAllocation && &b != &ws_rns && ws_rns.p) {
+      cudaGetLastError();
+      ws_rns.release();
+      e = b.ensure(bytes);
+    }
+    return e;
+  }
   std::mutex serve_mu;                      // guards creation of the serving engine
   tc::Server *server = nullptr;
 };

@@ -21,6 +21,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <vector>
+
 namespace tc {
 
 constexpr int MAX_BATCH = 32;
@@ -45,7 +47,7 @@ struct Work {
   const int4 *orb;     // (P, Q, R, 0) tile indices
   double *partial;     // [n_items][2]: the item's E_(T) part and its E[5]_ST (V r3(W)/D) part
   unsigned int *counter;
-  int *err;            // device error flag (0 = fine)
+  int *err;            // device error flag (0 = fine); err[1]: the FP64 tensor-core path's input flag
 };
 
 // The six permutations of three positions, in the order
@@ -60,7 +62,7 @@ __host__ __device__ constexpr int perm3(int s, int pos) {
 }
 __host__ __device__ constexpr bool perm3_even(int s) { return s == 0 || s == 3 || s == 4; }
 
-// ---------------------------------------------------------------- FP64 path
+// ---------------------------------------------------------------- FP64 path, DMMA kernel
 struct FpJob {
   Dims d;
   Inputs in;
@@ -172,6 +174,89 @@ cudaError_t launch_split_block(WtBatch &wb, EnBatch &eb, int S, int num_sms, cud
 // / ep to eb.  The nodes must run in the order wp[0], wp[1], wp[2], ep.
 cudaError_t split_block_params(WtBatch *wb, EnBatch &eb, int S, int num_sms, void **wargs, void **eargs,
                                cudaKernelNodeParams *wp, cudaKernelNodeParams *ep);
+
+// ---------------------------------------------------------------- FP64 path on the tensor cores (tc_rns.cu)
+// Geometry of one job: 128-row M tiles over the v^2 virtual pairs, K halves of
+// 8 over a virtual / an occupied index, N chunks over v.
+struct RnsGeom {
+  int o, v;
+  int mt;                // M tiles: ceil(v^2 / 128)
+  int hv, ho;            // K halves over a virtual / an occupied index (hv + ho is even)
+  int nch, nc;           // N chunks and their width (multiple of 16, <= 208)
+  int vc;                // innermost extent of the W buffer (v rounded up to 4)
+  int nb;                // triplets per block (capacity of the W buffer)
+};
+// Byte offsets inside a job's workspace: operand images, W buffer, the scale
+// search's norms, maxima and exponents, unit table, mask of occupied pairs.
+struct RnsLayout {
+  RnsGeom g;
+  size_t pa, pa2, hc, hc2, tb, hb, y, ra, rt, rb, rh, mx, ex, unit, need;
+  size_t total;
+};
+// Host tables of a triplet list.  A unit is one F GEMM of one triplet:
+// (triplet index << 3) | (half of K << 2) | F number.  unit holds the storing
+// launch's units (one per triplet), then the adding launch's; off[t] counts the
+// latter before triplet t.  need: occupied pairs whose operands are read.
+struct RnsTables {
+  std::vector<int> unit, off;
+  std::vector<unsigned char> need;
+};
+struct RnJob {           // one job's block of triplets in a GEMM launch
+  RnsGeom g;
+  const int4 *trip;      // the job's triplet table
+  const int *unit;       // the block's units
+  int t0, nu;            // first triplet of the block; number of units
+  const unsigned char *pa, *pa2, *hc, *hc2, *tb, *hb;
+  unsigned long long *y; // W buffer [triplet][a][b][vc], 64-bit fractions
+  long long item0;       // first global item of this job in the launch (set by the launcher)
+};
+struct RnBatch {
+  int njobs;
+  int stages, hps, acc;  // set by the launcher: pipeline stages, K halves of a stage, TMEM columns between the two accumulators (the
+                         // launch's widest N chunk: items of different jobs meet in the pipeline)
+  size_t slot;           // set by the launcher: stage stride in shared memory
+  long long total_items;
+  int *err;
+  RnJob job[MAX_BATCH];
+};
+struct RnEnJob {         // one job's block of triplets in an energy launch
+  Dims d;
+  int vc;
+  const int4 *trip, *orb;
+  const double *eps, *t1, *ovov;
+  const long long *y;
+  const int *ev, *uo, *sh;
+  double *partial;       // [n_items][2], slot t * items_per_trip + chunk
+  int t0, nt;
+  long long item0;
+};
+struct RnEnBatch {
+  int njobs;
+  long long total_items;
+  RnEnJob job[MAX_BATCH];
+};
+constexpr int RNS_GEMM_LAUNCHES = 2;       // storing, then adding
+constexpr int RNS_MIN_V = 8;
+// Whether the path covers the shape (K bound of the exact FP32 sums).
+bool rns_supported(int o, int v);
+RnsGeom rns_geom(int o, int v);
+RnsLayout rns_layout(int o, int v, int n_trip);
+RnsTables rns_tables(int o, const int4 *trip, int n);
+// Scales, operand images and unit table (all: every occupied pair's images,
+// else those t.need marks).  *flag (device) is set to 1 when the inputs leave
+// the range of the integer grid: the results are then not to be used.  t must
+// stay alive until st reaches the copies' end.
+cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, const RnsTables &t, bool all, int *flag,
+                            cudaStream_t st);
+int rns_prep_launches();
+// Jobs of triplets [t0, t0 + nt) for the two GEMM launches and the energy launch.
+void rns_block(const RnsLayout &L, void *ws, const Dims &d, const Inputs &in, const Work &w, const RnsTables &t, int t0,
+               int nt, RnJob *j0, RnJob *j1, RnEnJob *en);
+cudaError_t launch_rns_block(RnBatch *gb, RnEnBatch &eb, int num_sms, cudaStream_t st, cudaEvent_t w0 = nullptr,
+                             cudaEvent_t w1 = nullptr);
+// As split_block_params: gp[0], gp[1], ep must run in this order.
+cudaError_t rns_block_params(RnBatch *gb, RnEnBatch &eb, int num_sms, void **gargs, void **eargs,
+                             cudaKernelNodeParams *gp, cudaKernelNodeParams *ep);
 
 // ---------------------------------------------------------------- integrals from DF factors (tc_df.cu)
 // (ia|bd), (ia|jl) and (ia|jb) from B[nq][o+v][o+v] (Eq. 6) as exact digit

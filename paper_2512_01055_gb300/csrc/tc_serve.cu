@@ -7,8 +7,8 @@
 //     budget, allocates each job's device block from the stream-ordered pool,
 //     copies host inputs, uploads its work tables and (split path) builds its
 //     BF16 operand images, all on the job's own stream, then records an event;
-//   * the scheduler runs iterations: it picks a precision group (FP64 or split
-//     with s slices) round robin, gives every ready job of that group a slice
+//   * the scheduler runs iterations: it picks a precision group (FP64 on the
+//     tensor cores, FP64 on the DMMA kernel, or split with s slices) round robin, gives every ready job of that group a slice
 //     of its remaining work items (a fair share of an item budget sized to
 //     about iteration_ms), and replays the group's CUDA graph -- one
 //     persistent multi-job kernel over all those slices -- after updating the
@@ -23,6 +23,7 @@
 #include <deque>
 #include <memory>
 #include <mutex>
+#include <new>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -35,7 +36,8 @@ namespace tc {
 namespace {
 
 using Clock = std::chrono::steady_clock;
-constexpr int N_GROUPS = 4;               // 0: FP64, 1..3: split with 2..4 slices
+constexpr int N_GROUPS = 5;               // 0: FP64 (DMMA kernel), 1..3: split with 2..4 slices, 4: FP64 on the tensor cores
+constexpr int G_RNS = 4;
 
 enum class St { Queued, Prep, Ready, Done, Failed, Cancelled };
 
@@ -48,12 +50,14 @@ struct Req {
   const double *din[6] = {};              // device inputs used by the kernels
   const double *dB = nullptr;             // DF factors on the device
   char *mem = nullptr;                    // device block: [host inputs][DF integrals][DF scratch][workspace][split images]
-  size_t footprint = 0;
+  size_t footprint = 0, in_bytes = 0;     // all device bytes; bytes of the inputs as given
   size_t off_ints = 0, off_df = 0;        // DF jobs: assembled integrals and assembly scratch in the block
   Dims d{};
   plan::Layout L{};
   SplitLayout SL{};
-  size_t off_ws = 0, off_split = 0;
+  RnsLayout RL{};                         // FP64 on the tensor cores (group G_RNS)
+  RnsTables rt;
+  size_t off_ws = 0, off_split = 0;       // off_split: split images, or the FP64 path's residue images
   Work w{};
   cudaStream_t st = nullptr;
   cudaEvent_t ready = nullptr;
@@ -95,10 +99,13 @@ struct Server {
   double *d_out = nullptr;                // device: 4 doubles per job of a reduction (E, sum |e|, E[5]_ST)
   cudaGraph_t graph[N_GROUPS] = {};
   cudaGraphExec_t exec[N_GROUPS] = {};
-  cudaGraphNode_t knode[N_GROUPS][SPLIT_WT_LAUNCHES] = {};   // FP64 group: [0] only; split: the W-term chain
-  cudaGraphNode_t enode[N_GROUPS] = {};   // split groups: the energy launch after the W-term launches
-  double rate[N_GROUPS] = {3e7, 4e8, 3e8, 2e8};   // cost units per second (refined as iterations run)
+  cudaGraphNode_t knode[N_GROUPS][SPLIT_WT_LAUNCHES] = {};   // DMMA group: [0] only; others: the GEMM chain
+  cudaGraphNode_t enode[N_GROUPS] = {};   // the energy launch after the GEMM launches
+  double rate[N_GROUPS] = {3e7, 4e8, 3e8, 2e8, 1e9};   // cost units per second (refined as iterations run)
   int rr = 0;                             // round-robin cursor over groups
+  bool lingering[N_GROUPS] = {};          // a small batch of the group waits for more jobs (see batch_may_grow)
+  Clock::time_point t_linger[N_GROUPS];   // since when
+  int handing_in[N_GROUPS] = {};          // small jobs of the group whose host arrays tc_submit is copying
   int fault_alloc = 0, fault_stall_ms = 0;
   tc_serve_stats stats{};
   int fp64_per_sm = 1;
@@ -108,6 +115,7 @@ struct Server {
   void sched_loop();
   void start_prep(const std::shared_ptr<Req> &r);
   bool run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs);
+  bool batch_may_grow(int g, const std::vector<std::shared_ptr<Req>> &jobs) const;
   void finish(std::vector<std::shared_ptr<Req>> &done);
   void fail_job(const std::shared_ptr<Req> &r, tc_status s);
 };
@@ -115,6 +123,15 @@ struct Server {
 namespace {
 
 int group_of(int prec, int slices) { return prec == TC_FP64 ? 0 : slices - 1; }
+int gemm_launches(int g) { return g == 0 ? 1 : g == G_RNS ? RNS_GEMM_LAUNCHES : SPLIT_WT_LAUNCHES; }
+
+// Work units and their cost: one orbit's worth of K values; a unit is an item
+// of the DMMA kernel, else a whole triplet.
+void set_units(Req &q) {
+  const bool items = q.group == 0;
+  q.units = items ? q.d.n_items : q.d.n_trip;
+  q.cost_per_item = (double)(items ? q.d.orb_per_item : q.d.n_orb) * (q.v + 16.0 * ((q.o + 15) / 16));
+}
 
 }  // namespace
 
@@ -156,6 +173,18 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
   cudaError_t e = cudaSuccess;
   if (q.inject_alloc_fault) e = cudaErrorMemoryAllocation;
   if (e == cudaSuccess) e = cudaMallocAsync((void **)&q.mem, q.footprint, q.st);
+  if (e == cudaErrorMemoryAllocation && !q.inject_alloc_fault && q.group == G_RNS) {
+    // no room for the residue images: the job runs on the DMMA kernel
+    cudaGetLastError();
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      reserved -= q.RL.total;
+      q.footprint -= q.RL.total;
+      q.group = 0;
+      set_units(q);
+    }
+    e = cudaMallocAsync((void **)&q.mem, q.footprint, q.st);
+  }
   if (e != cudaSuccess) {
     q.mem = nullptr;
     std::lock_guard<std::mutex> lk(mu);
@@ -212,14 +241,23 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
   q.w.partial = (double *)(base + q.L.partial);
   q.w.counter = (unsigned *)(base + q.L.counter);
   q.w.err = (int *)(base + q.L.counter + sizeof(unsigned));
-  cudaMemsetAsync(q.w.counter, 0, 2 * sizeof(unsigned), q.st);
+  cudaMemsetAsync(q.w.counter, 0, 3 * sizeof(unsigned), q.st);
+  const Inputs in{q.din[0], q.din[1], q.din[2], q.din[3], q.din[4], q.din[5]};
+  int out_of_range = 0;
   if (split) {
-    const Inputs in{q.din[0], q.din[1], q.din[2], q.din[3], q.din[4], q.din[5]};
     launch_split_prep(q.SL, in, q.mem + q.off_split, q.st);
+  } else if (q.group == G_RNS) {
+    q.rt = rns_tables(q.o, tab.data(), q.d.n_trip);
+    launch_rns_prep(q.RL, in, q.mem + q.off_split, q.rt, true, q.w.err + 1, q.st);
+    cudaMemcpyAsync(&out_of_range, q.w.err + 1, sizeof(int), cudaMemcpyDeviceToHost, q.st);
   }
   cudaEventRecord(q.ready, q.st);
   e = cudaStreamSynchronize(q.st);        // the copies read the job's host vectors
   std::lock_guard<std::mutex> lk(mu);
+  if (out_of_range) {                     // beyond the integer grid: the DMMA kernel
+    q.group = 0;
+    set_units(q);
+  }
   for (auto &h : q.host) std::vector<double>().swap(h);
   if (e != cudaSuccess) {
     fail_job(r, TC_ECUDA);
@@ -274,8 +312,8 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
     std::vector<int> still;
     for (int j : open) {
       Req &q = *jobs[j];
-      // split jobs run at most one block of triplets (the W buffer) per launch
-      const long long cap = g == 0 ? q.units : q.SL.g.nb;
+      // jobs of the GEMM groups run at most one block of triplets (the W buffer) per launch
+      const long long cap = g == 0 ? q.units : g == G_RNS ? q.RL.g.nb : q.SL.g.nb;
       const long long rem = std::min(q.units - q.next_item, cap) - take[j];
       const long long want = std::max<long long>(1, (long long)(share / q.cost_per_item));
       const long long t = std::min(rem, want);
@@ -296,6 +334,8 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
   static thread_local FpBatch fb;
   static thread_local WtBatch wb[SPLIT_WT_LAUNCHES];
   static thread_local EnBatch eb;
+  static thread_local RnBatch gb[RNS_GEMM_LAUNCHES];
+  static thread_local RnEnBatch reb;
   long long total = 0;
   double cost = 0;
   cudaError_t e = cudaSuccess;
@@ -313,6 +353,17 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
     fb.total_items = total;
     const long long grid = std::min<long long>((long long)ctx->num_sms * fp64_per_sm, total);
     fp64_node_params(fb, (int)grid, args, &kp[0]);
+  } else if (g == G_RNS) {
+    gb[0].njobs = gb[1].njobs = reb.njobs = nj;
+    gb[0].err = gb[1].err = d_err;
+    for (int j = 0; j < nj; ++j) {
+      Req &q = *jobs[j];
+      const Inputs in{q.din[0], q.din[1], q.din[2], q.din[3], q.din[4], q.din[5]};
+      rns_block(q.RL, q.mem + q.off_split, q.d, in, q.w, q.rt, (int)q.next_item, (int)take[j], &gb[0].job[j],
+                &gb[1].job[j], &reb.job[j]);
+      cost += take[j] * q.cost_per_item;
+    }
+    e = rns_block_params(gb, reb, ctx->num_sms, args, eargs, kp, &ep);
   } else {
     wb[0] = WtBatch{};
     eb = EnBatch{};
@@ -332,7 +383,8 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
   if (e != cudaSuccess) return false;
   if (!exec[g]) {
     // the group's graph: FP64, [zero the work counter] -> [multi-job kernel];
-    // split, [W-term F0] -> [F1] -> [F2] -> [energy]
+    // split, [W-term F0] -> [F1] -> [F2] -> [energy]; FP64 on the tensor
+    // cores, [storing GEMM] -> [adding GEMM] -> [energy]
     e = cudaGraphCreate(&graph[g], 0);
     cudaGraphNode_t mnode = nullptr;
     if (e == cudaSuccess && g == 0) {
@@ -346,15 +398,15 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
     }
     if (e == cudaSuccess) e = cudaGraphAddKernelNode(&knode[g][0], graph[g], mnode ? &mnode : nullptr, mnode ? 1 : 0, &kp[0]);
     if (g != 0) {
-      for (int f = 1; f < SPLIT_WT_LAUNCHES && e == cudaSuccess; ++f)
+      for (int f = 1; f < gemm_launches(g) && e == cudaSuccess; ++f)
         e = cudaGraphAddKernelNode(&knode[g][f], graph[g], &knode[g][f - 1], 1, &kp[f]);
-      if (e == cudaSuccess) e = cudaGraphAddKernelNode(&enode[g], graph[g], &knode[g][SPLIT_WT_LAUNCHES - 1], 1, &ep);
+      if (e == cudaSuccess) e = cudaGraphAddKernelNode(&enode[g], graph[g], &knode[g][gemm_launches(g) - 1], 1, &ep);
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&exec[g], graph[g], 0);
   } else {
     e = cudaGraphExecKernelNodeSetParams(exec[g], knode[g][0], &kp[0]);
     if (g != 0) {
-      for (int f = 1; f < SPLIT_WT_LAUNCHES && e == cudaSuccess; ++f)
+      for (int f = 1; f < gemm_launches(g) && e == cudaSuccess; ++f)
         e = cudaGraphExecKernelNodeSetParams(exec[g], knode[g][f], &kp[f]);
       if (e == cudaSuccess) e = cudaGraphExecKernelNodeSetParams(exec[g], enode[g], &ep);
     }
@@ -416,6 +468,28 @@ void Server::finish(std::vector<std::shared_ptr<Req>> &done) {
   }
 }
 
+// Whether the ready jobs of group g are less than a quarter of an iteration's
+// work while a small job of the same group is being handed in, prepared or
+// about to be admitted: one launch over both costs little more than a launch
+// over one.  Caller holds mu.
+constexpr size_t SMALL = (size_t)64 << 20;                 // inputs of a job copied and prepared within milliseconds
+bool Server::batch_may_grow(int g, const std::vector<std::shared_ptr<Req>> &jobs) const {
+  double cost = 0;
+  for (auto &r : jobs) cost += (double)(r->units - r->next_item) * r->cost_per_item;
+  if (cost > 0.25e-3 * ctx->iteration_ms * rate[g] || (int)jobs.size() >= MAX_BATCH) return false;
+  if (handing_in[g] > 0) return true;
+  for (auto &r : active)
+    if (r->state == St::Prep && r->group == g && r->in_bytes <= SMALL) return true;
+  size_t room = ctx->budget - std::min(ctx->budget, reserved);
+  int slots = ctx->max_inflight - (int)active.size();
+  for (auto &r : queue) {
+    if (slots-- <= 0 || r->footprint > room || r->in_bytes > SMALL) break;
+    if (r->group == g) return true;
+    room -= r->footprint;
+  }
+  return false;
+}
+
 void Server::sched_loop() {
   cudaSetDevice(ctx->device);
   std::unique_lock<std::mutex> lk(mu);
@@ -440,24 +514,37 @@ void Server::sched_loop() {
         ++a;
       }
     }
-    // pick the next group (round robin) that has ready work
+    // pick the next group (round robin) that has ready work and whose batch is
+    // not about to grow; it waits for that a few iterations' time at most
     std::vector<std::shared_ptr<Req>> jobs;
     int g = -1;
+    bool waits = false;
     for (int k = 0; k < N_GROUPS && g < 0; ++k) {
       const int gg = (rr + k) % N_GROUPS;
       for (auto &r : active)
         if (r->group == gg && r->state == St::Ready && r->next_item < r->units && (int)jobs.size() < MAX_BATCH)
           jobs.push_back(r);
-      if (!jobs.empty()) g = gg;
+      if (jobs.empty()) continue;
+      if (batch_may_grow(gg, jobs)) {
+        const auto now = Clock::now();
+        if (!lingering[gg]) { lingering[gg] = true; t_linger[gg] = now; }
+        if (now - t_linger[gg] < std::chrono::milliseconds(4 * ctx->iteration_ms)) {
+          waits = true;
+          jobs.clear();
+          continue;
+        }
+      }
+      g = gg;
     }
     // jobs with no items at all (o = 1 or v too small to matter) complete directly
     std::vector<std::shared_ptr<Req>> done;
     for (auto &r : active)
       if (r->state == St::Ready && r->next_item >= r->units) { done.push_back(r); r->state = St::Prep; }
     if (g < 0 && done.empty()) {
-      cv_sched.wait_for(lk, std::chrono::milliseconds(2));
+      cv_sched.wait_for(lk, std::chrono::microseconds(waits ? 500 : 2000));
       continue;
     }
+    if (g >= 0) lingering[g] = false;
     rr = (g < 0 ? rr : g) + 1;
     lk.unlock();
     if (g >= 0) {
@@ -551,10 +638,16 @@ tc_status tc_submit(tc_ctx *ctx, const tc_job *job, uint64_t *ticket) {
               : tc::plan::make_dims(o, v, tc::fp64_tile());
   r->L = tc::plan::make_layout(r->d);
   if (split) r->SL = tc::split_layout(o, v, slices);
+  // FP64 on the tensor cores by the rule of the blocking entry points
+  if (!split && r->d.n_trip > 0 && tc::rns_supported(o, v)) {
+    r->RL = tc::rns_layout(o, v, r->d.n_trip);
+    if (r->RL.total <= ctx->budget / 4) r->group = tc::G_RNS;
+    else r->RL = tc::RnsLayout{};
+  }
   r->nq = job->nq;
   const size_t O = o, V = v, NB = (size_t)job->nq * (O + V) * (O + V);
   const size_t ints_b = sizeof(double) * (O * V * V * V + O * V * O * O + O * V * O * V);
-  // [host inputs][DF integrals][DF scratch][workspace][split images]
+  // [host inputs][DF integrals][DF scratch][workspace][split or residue images]
   const size_t in_b = r->dev_inputs ? 0
                       : tc::plan::align256(r->nq > 0 ? sizeof(double) * (O + V + O * V + O * O * V * V + NB)
                                                      : tc::plan::input_bytes(o, v));
@@ -562,10 +655,13 @@ tc_status tc_submit(tc_ctx *ctx, const tc_job *job, uint64_t *ticket) {
   r->off_df = r->off_ints + (r->nq > 0 ? tc::plan::align256(ints_b) : 0);
   r->off_ws = r->off_df + (r->nq > 0 ? tc::plan::align256(tc::df_scratch_bytes(o, v, r->nq)) : 0);
   r->off_split = r->off_ws + r->L.total;
-  r->footprint = r->off_split + r->SL.total;
-  // cost units: one orbit's worth of K values; a split unit is a whole triplet
-  r->units = split ? r->d.n_trip : r->d.n_items;
-  r->cost_per_item = (double)(split ? r->d.n_orb : r->d.orb_per_item) * (v + 16.0 * ((o + 15) / 16));
+  r->footprint = r->off_split + r->SL.total + r->RL.total;
+  r->in_bytes = r->nq > 0 ? sizeof(double) * (O * O * V * V + NB) : tc::plan::input_bytes(o, v);
+  if (r->footprint > ctx->budget && r->group == tc::G_RNS) {
+    r->footprint -= r->RL.total;
+    r->group = 0;
+  }
+  tc::set_units(*r);
   if (r->footprint > ctx->budget) return TC_ENOMEM;
   const double *src[6] = {job->eps, job->t1, job->t2, job->ints.ovvv, job->ints.ovoo, job->ints.ovov};
   const size_t n[6] = {O + V, O * V, O * O * V * V, O * V * V * V, O * V * O * O, O * V * O * V};
@@ -573,11 +669,27 @@ tc_status tc_submit(tc_ctx *ctx, const tc_job *job, uint64_t *ticket) {
   if (r->dev_inputs) {
     for (int a = 0; a < narr; ++a) r->din[a] = src[a];
     if (r->nq > 0) r->dB = job->B;
-  } else {
-    for (int a = 0; a < narr; ++a) r->host[a].assign(src[a], src[a] + n[a]);
-    if (r->nq > 0) r->host[3].assign(job->B, job->B + NB);
   }
   if (cudaEventCreateWithFlags(&r->ready, cudaEventDisableTiming) != cudaSuccess) return TC_ECUDA;
+  const bool told = !r->dev_inputs && r->in_bytes <= tc::SMALL;   // the scheduler knows of it during the copies
+  const int group = r->group;
+  if (told) {
+    std::lock_guard<std::mutex> lk(s->mu);
+    ++s->handing_in[group];
+  }
+  if (!r->dev_inputs) {
+    try {
+      for (int a = 0; a < narr; ++a) r->host[a].assign(src[a], src[a] + n[a]);
+      if (r->nq > 0) r->host[3].assign(job->B, job->B + NB);
+    } catch (const std::bad_alloc &) {
+      if (told) {
+        std::lock_guard<std::mutex> lk(s->mu);
+        --s->handing_in[group];
+      }
+      cudaEventDestroy(r->ready);
+      return TC_ENOMEM;
+    }
+  }
   r->res.o = o;
   r->res.v = v;
   r->res.prec = prec;
@@ -585,6 +697,7 @@ tc_status tc_submit(tc_ctx *ctx, const tc_job *job, uint64_t *ticket) {
   r->t_submit = tc::Clock::now();
   {
     std::lock_guard<std::mutex> lk(s->mu);
+    if (told) --s->handing_in[group];
     if ((int)s->queue.size() >= ctx->max_queue) {
       cudaEventDestroy(r->ready);
       return TC_EBUSY;
