@@ -68,8 +68,8 @@ constexpr int MROWS = 128;
 constexpr int A_HALF = MROWS * 16;           // bytes of one A half (8 K values)
 constexpr int HPS_MAX = 16;                  // most K halves of a pipeline stage
 constexpr int NCMAX = 208;                   // widest N chunk
-constexpr int REG_COLS = 80;                 // columns of a drain thread whose sums live in registers
-constexpr int TM_COLS = NCMAX / 2 - REG_COLS;// and in TMEM
+constexpr int REG_UNITS = 10;                // most units of 8 columns of a drain thread whose sums live in registers
+constexpr int TM_COLS = NCMAX / 2 - 8 * REG_UNITS;   // columns whose sums live in TMEM
 constexpr int TM_BASE = 512 - 4 * TM_COLS;   // first TMEM column of those sums (two halves, two words)
 constexpr int MAX_STAGES = 10;
 constexpr int NPROD = 3;
@@ -78,7 +78,7 @@ constexpr int DRAIN_WARPS = 8;
 constexpr int SMEM_DYN_MAX = 232448 - 2048;
 constexpr int NT = 8;                        // tile edge of the energy orbits
 constexpr int NT2 = NT * NT, NT3 = NT2 * NT;
-constexpr int EN_THREADS = 128, EN_CTAS = 4;   // per CTA, CTAs per SM
+constexpr int EN_THREADS = 128, EN_CTAS = 5;   // per CTA, CTAs per SM
 
 constexpr int ERR_TIMEOUT_FULL = 11, ERR_TIMEOUT_EMPTY = 12, ERR_TIMEOUT_ACCFULL = 13,
               ERR_TIMEOUT_ACCEMPTY = 14, ERR_TIMEOUT_TEARDOWN = 15;
@@ -583,11 +583,14 @@ __device__ __forceinline__ void add_frac(unsigned long long &acc, uint32_t u, co
 // m_l and added to the 64-bit sums.  The 64-bit multiply-add is the dear part
 // (8.4 of 12.7 clocks a column and warp), so moduli go in pairs: the first
 // (MODE 0) only packs its residues into bytes, the second (MODE 1) forms the
-// pair's 17-bit residue and adds that (9 clocks a column and modulus); MODE 2
-// is a modulus alone.  Columns whose sums live in TMEM always take that form.
-template <int MODE>
+// pair's 17-bit residue and adds that; MODE 2 is a modulus alone.  Columns
+// whose sums live in TMEM always take that form.  UN, the units of 8 columns in
+// registers, is fixed at compile time and columns behind the chunk are reduced
+// along: a test around every unit costs more (18.5 clocks a column and modulus
+// instead of 11.7).
+template <int MODE, int UN>
 __device__ __forceinline__ void drain_product(int l, int my, uint32_t tacc, uint32_t tmp,
-                                              unsigned long long (&part)[REG_COLS], uint32_t (&pk)[REG_COLS / 4]) {
+                                              unsigned long long (&part)[8 * UN], uint32_t (&pk)[2 * UN]) {
   ModConst mc;
   mc.inv = pack2(RC.inv[l]);
   mc.neg = pack2(RC.neg[l]);
@@ -602,9 +605,9 @@ __device__ __forceinline__ void drain_product(int l, int my, uint32_t tacc, uint
   tmem_ld8(tacc, c[0]);
   tmem_wait_ld8(c[0]);
 #pragma unroll
-  for (int u = 0; u < REG_COLS / 8; ++u) {
-    if (u < my) {
-      if (u + 1 < my && u + 1 < REG_COLS / 8) tmem_ld8(tacc + 8 * (u + 1), c[(u + 1) & 1]);
+  for (int u = 0; u < UN; ++u) {
+    {
+      if (u + 1 < UN) tmem_ld8(tacc + 8 * (u + 1), c[(u + 1) & 1]);
       const float (&x)[8] = c[u & 1];
       if (MODE == 0) {
 #pragma unroll
@@ -629,16 +632,16 @@ __device__ __forceinline__ void drain_product(int l, int my, uint32_t tacc, uint
           add_frac(part[8 * u + e + 1], u1, mc);
         }
       }
-      tmem_wait_ld8(c[(u + 1) & 1]);
+      if (u + 1 < UN) tmem_wait_ld8(c[(u + 1) & 1]);
     }
   }
-  if (my > REG_COLS / 8) {
+  if (UN == REG_UNITS && my > UN) {
     ModConst ms = mc;
     ms.ilo = (uint32_t)RC.I[l];
     ms.ihi = (uint32_t)(RC.I[l] >> 32);
 #pragma unroll 1
-    for (int u = REG_COLS / 8; u < my; ++u) {
-      const uint32_t ts = tmp + 16 * (uint32_t)(u - REG_COLS / 8);
+    for (int u = UN; u < my; ++u) {
+      const uint32_t ts = tmp + 16 * (uint32_t)(u - UN);
       float x[8];
       uint32_t plo[8] = {}, phi[8] = {};
       tmem_ld8(tacc + 8 * u, x);
@@ -667,6 +670,7 @@ __device__ __forceinline__ void drain_product(int l, int my, uint32_t tacc, uint
   }
 }
 
+template <int UN>
 __global__ void __launch_bounds__(THREADS, 1)
 rns_gemm_kernel(const __grid_constant__ RnBatch B) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -813,12 +817,27 @@ rns_gemm_kernel(const __grid_constant__ RnBatch B) {
             const uint32_t at = (sbase + (uint32_t)stage * slot) >> 4;
             const uint64_t da = da0 + at, db = db0 + at;
             if (el) {
-              const int n = min(B.hps, H - h0) / 2;
-#pragma unroll
-              for (int k = 0; k < HPS_MAX / 2; ++k)
-                if (k < n)
-                  mma_bf16(d, da + (uint32_t)(k * (2 * A_HALF >> 4)), db + (uint32_t)k * 2 * nc, id,
-                           (h0 == 0 && k == 0) ? 0u : 1u);
+              // the stage's K blocks in straight runs of 4, 2 and 1 (a test
+              // around every MMA would cost half an MMA's time each)
+              constexpr uint32_t SA = 2 * A_HALF >> 4;
+              const uint32_t SB = 2 * nc;
+              int n = min(B.hps, H - h0) / 2;
+              uint64_t xa = da, xb = db;
+              uint32_t acc = h0 > 0 ? 1u : 0u;
+              for (; n >= 4; n -= 4, xa += 4 * SA, xb += 4 * SB, acc = 1u) {
+                mma_bf16(d, xa, xb, id, acc);
+                mma_bf16(d, xa + SA, xb + SB, id, 1u);
+                mma_bf16(d, xa + 2 * SA, xb + 2 * SB, id, 1u);
+                mma_bf16(d, xa + 3 * SA, xb + 3 * SB, id, 1u);
+              }
+              if (n & 2) {
+                mma_bf16(d, xa, xb, id, acc);
+                mma_bf16(d, xa + SA, xb + SB, id, 1u);
+                xa += 2 * SA;
+                xb += 2 * SB;
+                acc = 1u;
+              }
+              if (n & 1) mma_bf16(d, xa, xb, id, acc);
               mma_commit(&empty_bar[stage]);
             }
             if (++stage == B.stages) { stage = 0; phase ^= 1u; }
@@ -853,17 +872,17 @@ rns_gemm_kernel(const __grid_constant__ RnBatch B) {
       const RnJob &J = B.job[jc];
       const int nc = J.g.nc, my = nc / 16;            // units of 8 columns of this thread
       const uint32_t c0 = (uint32_t)(hsel * (nc / 2));
-      unsigned long long part[REG_COLS];
+      unsigned long long part[8 * UN];
 #pragma unroll
-      for (int e = 0; e < REG_COLS; ++e) part[e] = 0;
-      uint32_t pk[REG_COLS / 4] = {};
+      for (int e = 0; e < 8 * UN; ++e) part[e] = 0;
+      uint32_t pk[2 * UN] = {};
       // wait for product l, reduce it, hand its accumulator back
       auto product = [&](auto mode, int l) {
         const uint32_t buf = cnt & 1u;
         const bool got = mbar_wait(&accfull_bar[buf], (cnt >> 1) & 1u, &abort_flag, B.err, ERR_TIMEOUT_ACCFULL);
         if (!__all_sync(0xffffffffu, got)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        drain_product<decltype(mode)::value>(l, my, trow + buf * (uint32_t)B.acc + c0, tmp, part, pk);
+        drain_product<decltype(mode)::value, UN>(l, my, trow + buf * (uint32_t)B.acc + c0, tmp, part, pk);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(&accempty_bar[buf]);
@@ -902,7 +921,7 @@ rns_gemm_kernel(const __grid_constant__ RnBatch B) {
         }
       };
 #pragma unroll
-      for (int u = 0; u < REG_COLS / 8; ++u) {
+      for (int u = 0; u < UN; ++u) {
         if (u < my) {
           unsigned long long s8[8];
 #pragma unroll
@@ -911,8 +930,8 @@ rns_gemm_kernel(const __grid_constant__ RnBatch B) {
         }
       }
 #pragma unroll 1
-      for (int u = REG_COLS / 8; u < my; ++u) {
-        const uint32_t ts = tmp + 16 * (uint32_t)(u - REG_COLS / 8);
+      for (int u = UN; u < my; ++u) {
+        const uint32_t ts = tmp + 16 * (uint32_t)(u - UN);
         uint32_t plo[8], phi[8];
         tmem_ld8u(ts, plo);
         tmem_ld8u(ts + 8, phi);
@@ -952,6 +971,17 @@ __device__ __forceinline__ double recip(double x) {
   return ex - 523u <= 1000u ? rcp_fast(x) : 1.0 / x;
 }
 
+// A 128-bit integer as a double (rounded once).
+__device__ __forceinline__ double u128_double(unsigned __int128 x) {
+  unsigned long long h = (unsigned long long)(x >> 64);
+  const unsigned long long l = (unsigned long long)x;
+  if (h == 0) return (double)l;
+  const int z = __clzll((long long)h);
+  if (z) h = h << z | l >> (64 - z);
+  const double d = (double)(h | ((l << z) != 0));          // the low bits as a sticky bit
+  return __hiloint2double(__double2hiint(d) + ((64 - z) << 20), __double2loint(d));
+}
+
 // One CTA per item (triplet, chunk of consecutive orbits).  The FP64 pipe (two
 // lanes per SM and clock) bounds it, so the work per point is arranged for few
 // FP64 operations.  With x_n the W values of the even and y_n of the odd
@@ -959,8 +989,9 @@ __device__ __forceinline__ double recip(double x) {
 // Eq. 1 is br = 3 x_n - se + 2 d and 3 y_n - so - 2 d: integers, exact while
 // |W| < 2^59 units (14 standard deviations on data of uniform size; larger
 // values take the same formulas in FP64), converted once each.  Then
-// sum_s w_s br_s = (sum_s br_s^2) / 3 - 6 d^2; 45 FP64 operations a point in all.
-// Four small CTAs on an SM keep the pipe fed while one of them loads.
+// sum_s w_s br_s = (sum_s br_s^2) / 3 - 6 d^2, formed in 128-bit integers (the
+// integer pipes have room beside the FP64 pipe); 37 FP64 operations a point in all.
+// Five small CTAs on an SM keep the pipe fed while one of them loads.
 // Orbits with equal tiles list their canonical points (36 x 8 of 512 points for
 // two equal tiles, 120 for three), so no warp runs for points outside them.
 __global__ void __launch_bounds__(EN_THREADS, EN_CTAS)
@@ -1071,29 +1102,35 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
           w[2] = w[3] = w[2] + w[3];
           w[4] = w[5] = w[4] + w[5];
         }
-        double br[6], dd;
+        double br[6], n4;                          // n4 = 3 sum_s w_s br_s
         unsigned long long big = 0;
 #pragma unroll
         for (int s = 0; s < 6; ++s) big |= (unsigned long long)(w[s] + (1LL << 59)) >> 60;
         if (big == 0) {
           const long long se = w[0] + w[3] + w[4], so = w[1] + w[2] + w[5], dl = se - so;
           const long long be = 2 * dl - se, bo = -2 * dl - so;
+          unsigned __int128 q = 0;
 #pragma unroll
-          for (int s = 0; s < 6; ++s) br[s] = (double)(3 * w[s] + (perm3_even(s) ? be : bo));
-          dd = (double)dl;
+          for (int s = 0; s < 6; ++s) {
+            const long long b = 3 * w[s] + (perm3_even(s) ? be : bo);
+            br[s] = (double)b;
+            const unsigned long long x = (unsigned long long)(b < 0 ? -b : b);
+            q += (unsigned __int128)x * x;
+          }
+          const unsigned long long x = (unsigned long long)(dl < 0 ? -dl : dl);
+          n4 = u128_double(q - (unsigned __int128)x * x * 18);
         } else {
           double f[6];
 #pragma unroll
           for (int s = 0; s < 6; ++s) f[s] = (double)w[s];
           const double se = f[0] + f[3] + f[4], so = f[1] + f[2] + f[5];
-          dd = se - so;
+          n4 = 0.0;
 #pragma unroll
-          for (int s = 0; s < 6; ++s) br[s] = 3.0 * f[s] + (perm3_even(s) ? se - 2.0 * so : so - 2.0 * se);
+          for (int s = 0; s < 6; ++s) {
+            br[s] = 3.0 * f[s] + (perm3_even(s) ? se - 2.0 * so : so - 2.0 * se);
+            n4 = fma(3.0 * f[s], br[s], n4);
+          }
         }
-        double n4 = br[0] * br[0];
-#pragma unroll
-        for (int s = 1; s < 6; ++s) n4 = fma(br[s], br[s], n4);
-        n4 = fma(-18.0 * dd, dd, n4);              // 3 sum_s w_s br_s
         auto T = [&](int op, int pos) { return Ts[(op * 3 + pos) * NT + l3[pos]]; };
         auto G = [&](int op, int u, int x) {       // G of op at positions (u, x) of the point
           const int tp = u == 0 ? (x == 1 ? 0 : 2) : u == 1 ? (x == 0 ? 1 : 4) : (x == 0 ? 3 : 5);
@@ -1163,8 +1200,17 @@ constexpr int PREP_BLOCKS = 152 * 16, PREP_THREADS = 256;
 
 size_t rn_slot(int hps, int ncmax) { return (size_t)hps * (A_HALF + (size_t)ncmax * 16); }
 
-// Item offsets, shared-memory plan and grids of a GEMM batch and an energy batch.
-cudaError_t prepare(RnBatch *gb, RnEnBatch &eb, int num_sms, int *ggrid, int *egrid, size_t *smem) {
+using RnKernel = void (*)(RnBatch);
+
+// The GEMM kernel instance for a widest N chunk of ncmax columns.
+RnKernel rn_kernel(int ncmax) {
+  const int u = ncmax / 16;
+  return u <= 3 ? rns_gemm_kernel<3> : u <= 5 ? rns_gemm_kernel<5> : u <= 7 ? rns_gemm_kernel<7>
+       : u <= 9 ? rns_gemm_kernel<9> : rns_gemm_kernel<REG_UNITS>;
+}
+
+// Item offsets, shared-memory plan, grids and kernel instance of a GEMM batch and an energy batch.
+cudaError_t prepare(RnBatch *gb, RnEnBatch &eb, int num_sms, int *ggrid, int *egrid, size_t *smem, RnKernel *fn) {
   int ncmax = 16;
   for (int f = 0; f < RNS_GEMM_LAUNCHES; ++f) {
     RnBatch &b = gb[f];
@@ -1201,7 +1247,8 @@ cudaError_t prepare(RnBatch *gb, RnEnBatch &eb, int num_sms, int *ggrid, int *eg
   }
   eb.total_items = total;
   *egrid = (int)std::max<long long>(1, std::min<long long>((long long)EN_CTAS * num_sms, total));
-  return cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  *fn = rn_kernel(ncmax);
+  return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
 }
 
 }  // namespace
@@ -1351,12 +1398,13 @@ cudaError_t rns_block_params(RnBatch *gb, RnEnBatch &eb, int num_sms, void **gar
                              cudaKernelNodeParams *gp, cudaKernelNodeParams *ep) {
   int ggrid[RNS_GEMM_LAUNCHES], egrid = 1;
   size_t smem = 0;
-  const cudaError_t e = prepare(gb, eb, num_sms, ggrid, &egrid, &smem);
+  RnKernel fn = nullptr;
+  const cudaError_t e = prepare(gb, eb, num_sms, ggrid, &egrid, &smem, &fn);
   if (e != cudaSuccess) return e;
   for (int f = 0; f < RNS_GEMM_LAUNCHES; ++f) {
     gargs[f] = (void *)&gb[f];
     gp[f] = cudaKernelNodeParams{};
-    gp[f].func = (void *)rns_gemm_kernel;
+    gp[f].func = (void *)fn;
     gp[f].gridDim = dim3(ggrid[f]);
     gp[f].blockDim = dim3(THREADS);
     gp[f].sharedMemBytes = (unsigned)smem;
@@ -1374,7 +1422,8 @@ cudaError_t rns_block_params(RnBatch *gb, RnEnBatch &eb, int num_sms, void **gar
 cudaError_t launch_rns_block(RnBatch *gb, RnEnBatch &eb, int num_sms, cudaStream_t st, cudaEvent_t w0, cudaEvent_t w1) {
   int ggrid[RNS_GEMM_LAUNCHES], egrid = 1;
   size_t smem = 0;
-  cudaError_t e = prepare(gb, eb, num_sms, ggrid, &egrid, &smem);
+  RnKernel fn = nullptr;
+  cudaError_t e = prepare(gb, eb, num_sms, ggrid, &egrid, &smem, &fn);
   if (e != cudaSuccess) return e;
   if (w0 && (e = cudaEventRecord(w0, st)) != cudaSuccess) return e;
   // programmatic launches, as launch_split_block: each kernel waits for its
@@ -1390,7 +1439,7 @@ cudaError_t launch_rns_block(RnBatch *gb, RnEnBatch &eb, int num_sms, cudaStream
   cfg.dynamicSmemBytes = smem;
   for (int f = 0; f < RNS_GEMM_LAUNCHES; ++f) {
     cfg.gridDim = dim3(ggrid[f]);
-    if ((e = cudaLaunchKernelEx(&cfg, rns_gemm_kernel, gb[f])) != cudaSuccess) return e;
+    if ((e = cudaLaunchKernelEx(&cfg, fn, gb[f])) != cudaSuccess) return e;
   }
   if (w1 && (e = cudaEventRecord(w1, st)) != cudaSuccess) return e;
   cfg.gridDim = dim3(egrid);
