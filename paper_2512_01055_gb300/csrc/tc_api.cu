@@ -146,7 +146,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
     TC_CUDA(ctx, cudaEventRecord(ctx->pev[0], st));
     TC_CUDA(ctx, tc::launch_split_prep_common(SL, in, ctx->ws_split.p, st));
     TC_CUDA(ctx, cudaEventRecord(ctx->pev[1], st));
-    launches += tc::split_prep_launches() - tc::split_prep_range_launches();
+    launches += tc::split_prep_common_launches();
   } else if (split) {
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
     TC_CUDA(ctx, tc::launch_split_prep(SL, in, ctx->ws_split.p, st));
@@ -157,7 +157,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[2], st));
     TC_CUDA(ctx, tc::launch_rns_prep(RL, in, ctx->ws_rns.p, rt, subset == nullptr, w.err + 1, st));
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[3], st));
-    launches += tc::rns_prep_launches();
+    launches += tc::rns_prep_launches(o, v);
   }
   if (d.n_items > 0) {
     TC_CUDA(ctx, cudaEventRecord(ctx->ev[0], st));

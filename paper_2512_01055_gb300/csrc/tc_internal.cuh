@@ -157,6 +157,7 @@ cudaError_t launch_split_prep(const SplitLayout &L, const Inputs &in, void *ws, 
 cudaError_t launch_split_prep_common(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st);
 cudaError_t launch_split_prep_range(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st, int p0, int p1);
 int split_prep_launches();
+int split_prep_common_launches();
 int split_prep_range_launches();
 WtJob wt_job(const SplitLayout &L, const void *ws, const int4 *trip, int t0, int nt);
 // Energy job of triplets [t0, t0 + nt); encodes its tensor map (driver entry point).
@@ -248,7 +249,7 @@ RnsTables rns_tables(int o, const int4 *trip, int n);
 // stay alive until st reaches the copies' end.
 cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, const RnsTables &t, bool all, int *flag,
                             cudaStream_t st);
-int rns_prep_launches();
+int rns_prep_launches(int o, int v);
 // Jobs of triplets [t0, t0 + nt) for the two GEMM launches and the energy launch.
 void rns_block(const RnsLayout &L, void *ws, const Dims &d, const Inputs &in, const Work &w, const RnsTables &t, int t0,
                int nt, RnJob *j0, RnJob *j1, RnEnJob *en);

@@ -238,8 +238,8 @@ __device__ __forceinline__ int rel_exp(unsigned long long bits, int emax) {
   return min(max((emax - e) / 2, 0), 40);
 }
 
-// One block: virtual exponents.
-__global__ void rns_virtual_exps(int v, Scales s) {
+// Virtual exponents, by one CTA.
+__device__ void virtual_exps(int v, const Scales &s) {
   __shared__ unsigned long long m;
   if (threadIdx.x == 0) m = 0;
   __syncthreads();
@@ -252,10 +252,9 @@ __global__ void rns_virtual_exps(int v, Scales s) {
 // 4^e as a double (|e| <= 500)
 __device__ __forceinline__ double pow4(int e) { return __longlong_as_double((long long)(1023 + 2 * e) << 52); }
 
-// Largest row norm of each occupied orbital after the virtual exponents.
-__global__ void rns_occ_norms(int o, int v, Scales s) {
+// Largest row norm of occupied orbital p after the virtual exponents.
+__device__ void occ_norms(int p, int v, const Scales &s) {
   const long long vv = (long long)v * v;
-  const int p = blockIdx.y;
   unsigned long long b = 0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < vv; e += (long long)gridDim.x * blockDim.x) {
     const double a = s.ra[p * vv + e] * pow4(s.ev[e / v] + s.ev[e % v]);
@@ -268,13 +267,12 @@ __global__ void rns_occ_norms(int o, int v, Scales s) {
 
 __device__ __forceinline__ int occ_exp(const Scales &s, int o, int p) {
   unsigned long long m = 0;
-  for (int q = 0; q < o; ++q) m = max(m, s.no[q]);
-  return rel_exp(s.no[p], m ? ilog2d(__longlong_as_double((long long)m)) : 0);
+  for (int q = 0; q < o; ++q) m = max(m, __ldcg(s.no + q));
+  return rel_exp(__ldcg(s.no + p), m ? ilog2d(__longlong_as_double((long long)m)) : 0);
 }
 
 // Largest scaled squared norms of the four operands.
-__global__ void rns_max_norms(int o, int v, Scales s) {
-  extern __shared__ int uo[];
+__device__ void max_norms(int o, int v, const Scales &s, int *uo) {
   for (int p = threadIdx.x; p < o; p += blockDim.x) {
     uo[p] = occ_exp(s, o, p);
     if (blockIdx.x == 0) s.uo[p] = uo[p];
@@ -309,11 +307,11 @@ __global__ void rns_max_norms(int o, int v, Scales s) {
 // share the grid (sa + sb = sah + sbh = SS); the pair with room to spare is
 // scaled down.  Arrays of zeros take shift 0; inputs whose norms leave
 // [2^-100, 2^100] or are not finite set the flag.
-__global__ void rns_shifts(Scales s) {
+__device__ void shifts(const Scales &s) {
   int i[4];
   bool any[4];
   for (int k = 0; k < 4; ++k) {
-    const unsigned long long b = s.mx[k];
+    const unsigned long long b = __ldcg(s.mx + k);
     any[k] = b != 0;
     const int e = any[k] ? (int)(b >> 52) - 1023 : 0;
     if (any[k] && (e < -200 || e > 200)) *s.flag = 1;
@@ -336,6 +334,28 @@ __global__ void rns_shifts(Scales s) {
   s.sh[2] = any[2] ? min(sb, BITS_B - i[2]) : sb;
   s.sh[3] = any[3] ? min(sbh, BITS_B - i[3]) : sbh;
   s.sh[4] = sa + sb;
+}
+
+__global__ void rns_virtual_exps(int v, Scales s) { virtual_exps(v, s); }
+__global__ void rns_occ_norms(int v, Scales s) { occ_norms(blockIdx.y, v, s); }
+__global__ void rns_max_norms(int o, int v, Scales s) {
+  extern __shared__ int uo[];
+  max_norms(o, v, s, uo);
+}
+__global__ void rns_shifts(Scales s) { shifts(s); }
+
+// All four steps by one CTA, for jobs where their launches take longer than
+// their work: up to SCALES_ONE rows of ovvv.
+constexpr long long SCALES_ONE = 1 << 16;
+__global__ void __launch_bounds__(1024) rns_scales_one(int o, int v, Scales s) {
+  extern __shared__ int uo[];
+  virtual_exps(v, s);
+  __syncthreads();
+  for (int p = 0; p < o; ++p) occ_norms(p, v, s);
+  __syncthreads();
+  max_norms(o, v, s, uo);
+  __syncthreads();
+  if (threadIdx.x == 0) shifts(s);
 }
 
 // ---------------------------------------------------------------- operand images
@@ -403,7 +423,7 @@ __device__ __forceinline__ uint4 residues8(const Limbs &x, int l, const unsigned
 // per image, with three limbs and packed FP32 for the reduction, took the
 // preparation of o=20 v=200 from 3.8 to 2.8 ms (9.6 GB of images).
 // need (may be NULL): only occupied indices p with need[p (o + 1)].
-__global__ void rns_image_a(bool vv, const double *__restrict__ src, RnsGeom G, Scales s,
+__device__ void rns_image_a(bool vv, const double *__restrict__ src, RnsGeom G, Scales s,
                             const unsigned char *__restrict__ need, unsigned char *__restrict__ out,
                             unsigned char *__restrict__ outT) {
   const int o = G.o, v = G.v, nh = vv ? G.hv : G.ho, kmax = vv ? v : o;
@@ -458,7 +478,7 @@ __global__ void rns_image_a(bool vv, const double *__restrict__ src, RnsGeom G, 
 // B images: row z, K f: t_rq^zf = t2[r][q][z][f] (vv), or K l: -(r z|q l) =
 // -ovoo[r][z][q][l]; rows or K values outside are zero.  One thread per (K
 // half, row).  need (may be NULL): only occupied pairs with need[r o + q].
-__global__ void rns_image_b(bool vv, const double *__restrict__ src, RnsGeom G, Scales s,
+__device__ void rns_image_b(bool vv, const double *__restrict__ src, RnsGeom G, Scales s,
                             const unsigned char *__restrict__ need, unsigned char *__restrict__ out) {
   const int o = G.o, v = G.v, rows = G.nc, nh = vv ? G.hv : G.ho, kmax = vv ? v : o;
   const size_t half_bytes = (size_t)rows * 16;
@@ -483,6 +503,17 @@ __global__ void rns_image_b(bool vv, const double *__restrict__ src, RnsGeom G, 
     const size_t step = (size_t)nh * half_bytes / sizeof(uint4);
 #pragma unroll 1
     for (int l = 0; l < RL; ++l) d[l * step] = residues8(lb, l, RC.cb, RC.hb[l]);
+  }
+}
+
+// All images in one launch, one task per blockIdx.y.
+__global__ void rns_images(RnsLayout L, Inputs in, Scales s, const unsigned char *__restrict__ need,
+                           unsigned char *__restrict__ b) {
+  switch (blockIdx.y) {
+    case 0: rns_image_a(true, in.ovvv, L.g, s, need, b + L.pa, b + L.pa2); break;
+    case 1: rns_image_b(true, in.t2, L.g, s, need, b + L.tb); break;
+    case 2: rns_image_a(false, in.t2, L.g, s, need, b + L.hc2, b + L.hc); break;
+    case 3: rns_image_b(false, in.ovoo, L.g, s, need, b + L.hb); break;
   }
 }
 
@@ -1329,7 +1360,7 @@ RnsTables rns_tables(int o, const int4 *trip, int n) {
   return t;
 }
 
-int rns_prep_launches() { return 9; }
+int rns_prep_launches(int o, int v) { return (long long)o * v * v <= SCALES_ONE ? 3 : 6; }
 
 cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, const RnsTables &t, bool all, int *flag,
                             cudaStream_t st) {
@@ -1342,15 +1373,18 @@ cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, cons
   if (e != cudaSuccess) return e;
   const unsigned char *need = all ? nullptr : (const unsigned char *)(b + L.need);
   rns_norms<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(in, g.o, g.v, s);
-  rns_virtual_exps<<<1, 512, 0, st>>>(g.v, s);
-  rns_occ_norms<<<dim3(16, g.o), 256, 0, st>>>(g.o, g.v, s);
-  rns_max_norms<<<152 * 2, 256, (size_t)g.o * sizeof(int), st>>>(g.o, g.v, s);
-  rns_shifts<<<1, 1, 0, st>>>(s);
+  if ((long long)g.o * g.v * g.v <= SCALES_ONE) {
+    rns_scales_one<<<1, 1024, (size_t)g.o * sizeof(int), st>>>(g.o, g.v, s);
+  } else {
+    rns_virtual_exps<<<1, 512, 0, st>>>(g.v, s);
+    rns_occ_norms<<<dim3(16, g.o), 256, 0, st>>>(g.v, s);
+    rns_max_norms<<<152 * 2, 256, (size_t)g.o * sizeof(int), st>>>(g.o, g.v, s);
+    rns_shifts<<<1, 1, 0, st>>>(s);
+  }
   unsigned char *ub = (unsigned char *)b;
-  rns_image_a<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(true, in.ovvv, g, s, need, ub + L.pa, ub + L.pa2);
-  rns_image_a<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(false, in.t2, g, s, need, ub + L.hc2, ub + L.hc);
-  rns_image_b<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(true, in.t2, g, s, need, ub + L.tb);
-  rns_image_b<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(false, in.ovoo, g, s, need, ub + L.hb);
+  const long long work = (long long)g.o * ((g.v + 7) / 8) * ((g.v + 3) / 4) * g.hv;   // warps of the largest task
+  const int blocks = (int)std::max<long long>(1, std::min<long long>(PREP_BLOCKS, (work + 7) / 8));
+  rns_images<<<dim3(blocks, 4), PREP_THREADS, 0, st>>>(L, in, s, need, ub);
   return cudaGetLastError();
 }
 

@@ -950,93 +950,121 @@ tc_energy_kernel(const __grid_constant__ EnBatch B) {
 
 // ---------------------------------------------------------------- operand images
 
-// One thread per (K half, row): reads 8 consecutive K values of one operand
-// row, splits them into S BF16 slices and writes 16 bytes per slice at the
-// row's place in the no-swizzle K-major half (core matrices of 8 rows x 16
-// bytes, 8-row groups 128 bytes apart).  An image is a sequence of halves,
-// each S slices of rows x 16 bytes; rows or K values outside the tensors are
-// zero.
-//   kind 0  A  [p][m][hv]        row (x, y), K f:  (p x | y f)            = ovvv[p][x][y][f]
-//   kind 1  A  [p][m][hv]        row (x, y), K f:  (p y | x f)            = ovvv[p][y][x][f]
-//   kind 2  A  [p][m][ho]        row (x, y), K l:  t_lp^xy = t_pl^yx      = t2[p][l][y][x]
-//   kind 3  A  [p][m][ho]        row (x, y), K l:  t_lp^yx = t_pl^xy      = t2[p][l][x][y]
-//   kind 4  B  [r][q][nc][hv]    row z,      K f:  t_rq^zf                = t2[r][q][z][f]
-//   kind 5  B  [r][q][nc][ho]    row z,      K l:  -(r z | q l)           = -ovoo[r][z][q][l]
-// (kinds 2 and 3 read t_lp^.. as t_pl^.. with the virtual pair swapped, which
-// keeps the reads coalesced).  Every kind's halves are ordered by the first
-// occupied index of the tensor they read (p, or r), so the threads of one
-// first-index range are the contiguous range [e_begin, e_end) of the image's
-// (half, row) index.
-__global__ void build_image(int kind, const double *__restrict__ src, SplitGeom G, long long e_begin,
-                            long long e_end, unsigned char *__restrict__ out) {
-  const int o = G.o, v = G.v, S = G.S;
-  const bool isA = kind < 4;
-  const int rows = isA ? MROWS : G.nc;
-  const int nh = (kind == 0 || kind == 1 || kind == 4) ? G.hv : G.ho;
-  const int kmax = (kind == 0 || kind == 1 || kind == 4) ? v : o;
-  const long long nhalf = isA ? (long long)o * G.mt * nh : (long long)o * o * G.nch * nh;
+// An image is a sequence of K halves, each S slices of rows x 16 bytes in the
+// no-swizzle K-major layout (core matrices of 8 rows x 16 bytes, 8-row groups
+// 128 bytes apart, so row r lies 16 r bytes into its slice); rows or K values
+// outside the tensors are zero.
+//   pa   A  [p][m][hv]        row (x, y), K f:  (p x | y f)            = ovvv[p][x][y][f]
+//   pa2  A  [p][m][hv]        row (x, y), K f:  (p y | x f)            = ovvv[p][y][x][f]
+//   hc   A  [p][m][ho]        row (x, y), K l:  t_lp^xy = t_pl^yx      = t2[p][l][y][x]
+//   hc2  A  [p][m][ho]        row (x, y), K l:  t_lp^yx = t_pl^xy      = t2[p][l][x][y]
+//   tb   B  [r][q][nc][hv]    row z,      K f:  t_rq^zf                = t2[r][q][z][f]
+//   hb   B  [r][q][nc][ho]    row z,      K l:  -(r z | q l)           = -ovoo[r][z][q][l]
+// Every image is ordered by the first occupied index of the tensor it reads.
+
+// The slices of 8 values, BF16, written to out + p step (and outT + p step) for
+// p < S.  x becomes a float pair (h, l) once, l rounded to odd (its last bit set
+// when bits are lost), so later roundings to fewer bits come out as from x
+// itself (Boldo and Melquiond): four FP64 operations, GB300's FP64 pipe being
+// 1/64 of its FP32 pipe, where taking every slice and residual in FP64 costs
+// three each.  A slice is the BF16 nearest to h + l: of their FP32 sum s, or
+// where s lies midway between two, of the side its rounding error (TwoSum)
+// points to; s minus the slice, exact, and that error are the next pair.
+__device__ __forceinline__ void write_slices(const double (&x)[8], int S, uint4 *out, uint4 *outT, size_t step) {
+  float h[8], l[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    h[u] = __double2float_rn(x[u]);
+    const double r = x[u] - (double)h[u];
+    l[u] = __double2float_rz(r);
+    if (__double2loint(r) & 0x1FFFFFFF) l[u] = __uint_as_float(__float_as_uint(l[u]) | 1u);
+  }
+  for (int p = 0; p < S; ++p) {
+    uint32_t b[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const float s = h[u] + l[u], t = s - h[u], er = (h[u] - (s - t)) + (l[u] - t);
+      const uint32_t bits = __float_as_uint(s);
+      b[u] = __bfloat16_as_ushort(__float2bfloat16_rn(s));
+      if ((bits & 0xFFFF) == 0x8000 && er != 0.f) b[u] = (bits >> 16) + (((__float_as_uint(er) ^ bits) >> 31) ^ 1u);
+      h[u] = s - __uint_as_float(b[u] << 16);
+      l[u] = er;
+    }
+    const uint4 q = make_uint4(b[0] | b[1] << 16, b[2] | b[3] << 16, b[4] | b[5] << 16, b[6] | b[7] << 16);
+    out[p * step] = q;
+    if (outT) outT[p * step] = q;
+  }
+}
+
+// A images of the occupied indices [p0, p1), both orders of the virtual pair
+// at once: the value of (x, y) goes to row (x, y) of out and row (y, x) of outT
+// (vv: ovvv into pa and pa2; else t2 into hc2 and hc).  A warp takes 8 x by 4 y,
+// so its stores cover 64 and 128 contiguous bytes; consecutive warps take
+// consecutive K halves of the same pairs.  The rows behind the last pair of the
+// last M tile are zeroed by the trailing warps.
+__device__ void image_a(bool vv, const double *__restrict__ src, const SplitGeom &G, int p0, int p1,
+                        unsigned char *__restrict__ out, unsigned char *__restrict__ outT) {
+  const int o = G.o, v = G.v, S = G.S, nh = vv ? G.hv : G.ho, kmax = vv ? v : o;
+  const int nx = (v + 7) / 8, ny = (v + 3) / 4, lane = threadIdx.x & 31;
+  const long long rows = (long long)v * v, per_p = (long long)nx * ny * nh;
+  const int tail = (int)(G.mt * (long long)MROWS - rows), tw = (tail + 31) / 32;
+  const long long np = p1 - p0, total = np * per_p + np * nh * tw, warps = (long long)gridDim.x * (blockDim.x >> 5);
+  auto at = [&](unsigned char *b, long long p, long long row, int h) {
+    return (uint4 *)(b + (((p * G.mt + row / MROWS) * nh + h) * S) * A_HALF + row % MROWS * 16);
+  };
+  const size_t step = A_HALF / sizeof(uint4);
+  for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < total; w += warps) {
+    if (w >= np * per_p) {
+      const long long e = w - np * per_p;
+      const int r = (int)(e % tw) * 32 + lane, h = (int)(e / tw % nh);
+      const long long p = p0 + e / tw / nh;
+      if (r < tail)
+        for (int q = 0; q < S; ++q) {
+          at(out, p, rows + r, h)[q * step] = make_uint4(0, 0, 0, 0);
+          at(outT, p, rows + r, h)[q * step] = make_uint4(0, 0, 0, 0);
+        }
+      continue;
+    }
+    const long long p = p0 + w / per_p, e = w % per_p;
+    const int h = (int)(e % nh), px = (int)(e / nh / ny), py = (int)(e / nh % ny);
+    const int x = px * 8 + (lane & 7), y = py * 4 + (lane >> 3);
+    if (x >= v || y >= v) continue;
+    double val[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = h * 8 + u;
+      val[u] = k >= kmax ? 0.0 : vv ? src[((p * v + x) * v + y) * v + k] : src[((p * o + k) * v + x) * v + y];
+    }
+    write_slices(val, S, at(out, p, (long long)x * v + y, h), at(outT, p, (long long)y * v + x, h), step);
+  }
+}
+
+// B images of the first occupied indices [p0, p1), one thread per (K half, row).
+__device__ void image_b(bool vv, const double *__restrict__ src, const SplitGeom &G, int p0, int p1,
+                        unsigned char *__restrict__ out) {
+  const int o = G.o, v = G.v, S = G.S, rows = G.nc, nh = vv ? G.hv : G.ho, kmax = vv ? v : o;
   const size_t half_bytes = (size_t)rows * 16;
-  const long long total = min(nhalf * rows, e_end);
-  const long long vv = (long long)v * v;
-  for (long long e = e_begin + blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
+  const long long per = (long long)o * G.nch * nh * rows;
+  for (long long e = per * p0 + blockIdx.x * (long long)blockDim.x + threadIdx.x; e < per * p1;
        e += (long long)gridDim.x * blockDim.x) {
     const int r = (int)(e % rows);
     const long long hb = e / rows;
     const int h = (int)(hb % nh);
-    const long long rest = hb / nh;
-    const int k0 = h * 8;
-    double x[8];
-    if (isA) {
-      const int m = (int)(rest % G.mt);
-      const long long p = rest / G.mt;
-      const long long row = (long long)m * MROWS + r;
-      const bool valid = row < vv;
-      const long long xi = valid ? row / v : 0, yi = valid ? row % v : 0;
+    const long long rest = hb / nh, pair = rest / G.nch, rr = pair / o, qq = pair % o;
+    const int z = (int)(rest % G.nch) * rows + r;
+    double val[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = k0 + u;
-        double val = 0.0;
-        if (valid && k < kmax) {
-          if (kind == 0)      val = src[((p * v + xi) * v + yi) * v + k];
-          else if (kind == 1) val = src[((p * v + yi) * v + xi) * v + k];
-          else if (kind == 2) val = src[((p * o + k) * v + yi) * v + xi];
-          else                val = src[((p * o + k) * v + xi) * v + yi];
-        }
-        x[u] = val;
-      }
-    } else {
-      const int nci = (int)(rest % G.nch);
-      const long long pair = rest / G.nch;               // r * o + q
-      const long long rr = pair / o, qq = pair % o;
-      const int z = nci * G.nc + r;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = k0 + u;
-        double val = 0.0;
-        if (z < v && k < kmax) {
-          if (kind == 4) val = src[((rr * o + qq) * v + z) * v + k];
-          else           val = -src[((rr * v + z) * o + qq) * o + k];
-        }
-        x[u] = val;
-      }
+    for (int u = 0; u < 8; ++u) {
+      const int k = h * 8 + u;
+      val[u] = z >= v || k >= kmax ? 0.0
+             : vv ? src[((rr * o + qq) * v + z) * v + k] : -src[((rr * v + z) * o + qq) * o + k];
     }
-    // position of row r in its half: 8-row group r/8, row r%8
-    const int off = (r >> 3) * 128 + (r & 7) * 16;
-    unsigned char *base = out + (size_t)hb * S * half_bytes + off;
-    for (int p = 0; p < S; ++p) {
-      __align__(16) __nv_bfloat16 b16[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        b16[u] = __double2bfloat16(x[u]);
-        x[u] -= (double)__bfloat162float(b16[u]);        // exact FP64 residual
-      }
-      *(uint4 *)(base + (size_t)p * half_bytes) = *(const uint4 *)b16;
-    }
+    write_slices(val, S, (uint4 *)(out + (size_t)hb * S * half_bytes + (size_t)r * 16), nullptr, half_bytes / sizeof(uint4));
   }
 }
 
 // FP32 copy of a [rows][cols] array with rows ld floats apart (zero beyond cols).
-__global__ void f32_rows(const double *__restrict__ in, long long rows, int cols, int ld, float *__restrict__ out) {
+__device__ void f32_rows(const double *__restrict__ in, long long rows, int cols, int ld, float *__restrict__ out) {
   const long long n = rows * ld;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     const long long r = e / ld;
@@ -1046,7 +1074,7 @@ __global__ void f32_rows(const double *__restrict__ in, long long rows, int cols
 }
 
 // Float pair of each value: out[e] = fl(x), out[n + e] = fl(x - fl(x)).
-__global__ void f32_hilo(const double *__restrict__ in, int n, float *__restrict__ out) {
+__device__ void f32_hilo(const double *__restrict__ in, int n, float *__restrict__ out) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
     const float h = (float)in[e];
     out[e] = h;
@@ -1058,7 +1086,7 @@ __global__ void f32_hilo(const double *__restrict__ in, int n, float *__restrict
 // out[0][p][u][q][w] = ovov[p][u][q][w], out[1][q][w][p][u] = ovov[p][u][q][w],
 // for the entries read from ovov rows p in [p0, p1) (ovov's first index: the
 // first index of out[0], the third of out[1]).
-__global__ void ovov_f32(const double *__restrict__ ovov, int o, int v, int vc, int p0, int p1,
+__device__ void ovov_f32(const double *__restrict__ ovov, int o, int v, int vc, int p0, int p1,
                          float *__restrict__ out) {
   const int np = p1 - p0;
   const long long half = (long long)o * v * o * vc, part = (long long)np * v * o * vc;
@@ -1085,6 +1113,24 @@ __global__ void ovov_f32(const double *__restrict__ ovov, int o, int v, int vc, 
       val = (float)(h == 0 ? ovov[(((long long)x0 * v + x1) * o + x2) * v + x3]
                            : ovov[(((long long)x2 * v + x3) * o + x0) * v + x1]);
     out[h * half + (((long long)x0 * v + x1) * o + x2) * vc + x3] = val;
+  }
+}
+
+// The whole preparation in one launch, task y0 + blockIdx.y: on small jobs the
+// nine launches it used to be took longer one after another (74 us at o=6 v=36)
+// than their work side by side.
+constexpr int PREP_RANGE_TASKS = 5, PREP_TASKS = 7;    // tasks of an index range; with those of t1 and eps
+__global__ void split_prep_kernel(const __grid_constant__ SplitLayout L, const __grid_constant__ Inputs in,
+                                  unsigned char *__restrict__ b, int p0, int p1, int y0) {
+  const SplitGeom &g = L.g;
+  switch (y0 + blockIdx.y) {
+    case 0: image_a(true, in.ovvv, g, p0, p1, b + L.pa, b + L.pa2); break;
+    case 1: image_b(true, in.t2, g, p0, p1, b + L.tb); break;
+    case 2: image_a(false, in.t2, g, p0, p1, b + L.hc2, b + L.hc); break;
+    case 3: image_b(false, in.ovoo, g, p0, p1, b + L.hb); break;
+    case 4: ovov_f32(in.ovov, g.o, g.v, g.vc, p0, p1, (float *)(b + L.ovovf)); break;
+    case 5: f32_rows(in.t1, g.o, g.v, g.vc, (float *)(b + L.t1f)); break;
+    case 6: f32_hilo(in.eps, g.o + g.v, (float *)(b + L.epsf)); break;
   }
 }
 
@@ -1229,45 +1275,37 @@ SplitLayout split_layout(int o, int v, int S) {
 }
 
 namespace {
-// (half, row) entries of image `kind` per value of its first occupied index.
-long long image_per_first(int kind, const SplitGeom &g) {
-  const int nh = (kind == 0 || kind == 1 || kind == 4) ? g.hv : g.ho;
-  return kind < 4 ? (long long)g.mt * nh * MROWS : (long long)g.o * g.nch * nh * g.nc;
+constexpr int PREP_THREADS = 256;
+// CTAs a task of one launch gets: two warps' worth of pairs each, at most 16 per SM.
+int prep_blocks(const SplitGeom &g, int np) {
+  const long long warps = (long long)np * ((g.v + 7) / 8) * ((g.v + 3) / 4) * g.hv;
+  return (int)std::max<long long>(1, std::min<long long>(152 * 16, (warps + 7) / 8));
 }
-constexpr int PREP_BLOCKS = 152 * 16, PREP_THREADS = 256;
 }  // namespace
 
 cudaError_t launch_split_prep_common(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st) {
-  const SplitGeom &g = L.g;
-  unsigned char *b = (unsigned char *)ws;
-  f32_rows<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(in.t1, g.o, g.v, g.vc, (float *)(b + L.t1f));
-  f32_hilo<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(in.eps, g.o + g.v, (float *)(b + L.epsf));
+  split_prep_kernel<<<dim3(64, PREP_TASKS - PREP_RANGE_TASKS), PREP_THREADS, 0, st>>>(L, in, (unsigned char *)ws, 0, 0,
+                                                                                      PREP_RANGE_TASKS);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_prep_range(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st, int p0,
                                     int p1) {
-  const SplitGeom &g = L.g;
-  if (p0 < 0 || p1 > g.o || p0 >= p1) return cudaErrorInvalidValue;
-  unsigned char *b = (unsigned char *)ws;
-  const size_t off[6] = {L.pa, L.pa2, L.hc, L.hc2, L.tb, L.hb};
-  const double *src[6] = {in.ovvv, in.ovvv, in.t2, in.t2, in.t2, in.ovoo};
-  for (int kind = 0; kind < 6; ++kind) {
-    const long long per = image_per_first(kind, g);
-    build_image<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(kind, src[kind], g, per * p0, per * p1, b + off[kind]);
-  }
-  ovov_f32<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(in.ovov, g.o, g.v, g.vc, p0, p1, (float *)(b + L.ovovf));
+  if (p0 < 0 || p1 > L.g.o || p0 >= p1) return cudaErrorInvalidValue;
+  split_prep_kernel<<<dim3(prep_blocks(L.g, p1 - p0), PREP_RANGE_TASKS), PREP_THREADS, 0, st>>>(
+      L, in, (unsigned char *)ws, p0, p1, 0);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_prep(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st) {
-  cudaError_t e = launch_split_prep_common(L, in, ws, st);
-  if (e != cudaSuccess) return e;
-  return launch_split_prep_range(L, in, ws, st, 0, L.g.o);
+  split_prep_kernel<<<dim3(prep_blocks(L.g, L.g.o), PREP_TASKS), PREP_THREADS, 0, st>>>(L, in, (unsigned char *)ws, 0,
+                                                                                       L.g.o, 0);
+  return cudaGetLastError();
 }
 
-int split_prep_launches() { return 9; }
-int split_prep_range_launches() { return 7; }
+int split_prep_launches() { return 1; }
+int split_prep_common_launches() { return 1; }
+int split_prep_range_launches() { return 1; }
 
 WtJob wt_job(const SplitLayout &L, const void *ws, const int4 *trip, int t0, int nt) {
   const unsigned char *b = (const unsigned char *)ws;
