@@ -60,9 +60,9 @@ typedef enum {
   TC_FP64 = 0,         /* FP64-accurate W, FP64 epilogue and sums.  W as exact integer products in residues on
                           the BF16 tensor cores: operands rounded once to a common power-of-two grid at least 2^-53
                           of their norms, W to 64 bits (an error below that of FP64 accumulation); or with FP64
-                          tensor-core (DMMA) tiles where the shape (o < 2, v < 8, K = 2v + 2o padded above 1024),
-                          the memory (the residue images take at most a quarter of the budget) or the inputs
-                          (infinities, NaN, norms outside 2^+-100) do not allow it */
+                          tensor-core (DMMA) tiles where the shape (o < 2, v < 9, K = 2v + 2o padded above 1024),
+                          the memory (budget and device) or the inputs (infinities, NaN, norms outside 2^+-100)
+                          do not allow it */
   TC_SPLIT_BF16 = 1    /* W built from BF16 slices on tcgen05 tensor cores, FP32 accumulation;
                           V and the Eq. 1 bracket in FP32; D, 1/D, each point's quotient and
                           the sums over a work item in float pairs (~48 significant bits);
@@ -128,7 +128,8 @@ tc_status tc_init(tc_ctx **ctx, const tc_options *opt);
  * TC_SPLIT_BF16, <= 0 for the default; ignored for TC_FP64.  TC_FP64 holds
  * residue images of the operands (30 bytes per element of ovvv in each of two
  * orders) besides tc_workspace_bytes while the context's budget and the device
- * have room for them; they are given back when another call needs the memory.
+ * have room for them; they are given back after the call when they exceed a
+ * quarter of the budget, and when another call needs the memory.
  * e_ijk (optional, may be NULL): host array [o][o][o] that receives the
  * weighted contribution of each occupied triplet i >= j >= k at [i][j][k]
  * (E_(T) is their sum); entries with i < j or j < k are set to 0. */

@@ -91,12 +91,26 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   if (need > ctx->budget) return fail(ctx, TC_ENOMEM, "workspace %zu B exceeds budget %zu B", need, ctx->budget);
   TC_CUDA(ctx, ctx->grow(ctx->ws, L.total));
   if (split) TC_CUDA(ctx, ctx->grow(ctx->ws_split, SL.total));
-  // FP64: on the tensor cores where the path covers the shape, its workspace
-  // takes at most a quarter of the budget (the rest stays for the caller's own
-  // arrays) and the device has the room; else the DMMA kernel.
+  // FP64: on the tensor cores where the path covers the shape and the context's
+  // budget and the device have room for its workspace; else the DMMA kernel.
+  // A workspace above a quarter of the budget is given back after the call, and
+  // taken only where the work repays it: allocating and releasing 185 GB adds
+  // 0.8 s (4.3 ps a byte) to the 50 s of o=40 v=400, and the DMMA kernel does
+  // 0.9 flop per ps, so 12 v^4 flop a triplet against 10 flop a byte leaves a
+  // factor of 2.5 (the whole energy: 71 against 1.0 TFLOP/s).
   const tc::RnsLayout RL = split ? tc::RnsLayout{} : tc::rns_layout(o, v, d.n_trip);
-  bool rns = !split && !dmma && d.n_trip > 0 && tc::rns_supported(o, v) && RL.total <= ctx->budget / 4 &&
+  bool rns = !split && !dmma && d.n_trip > 0 && tc::rns_supported(o, v) &&
+             (RL.total <= ctx->budget / 4 || 12.0 * d.n_trip * v * v * v * v >= 10.0 * RL.total) &&
              need + RL.total + ctx->in_ovvv.cap + ctx->in_t2.cap + ctx->in_ovov.cap + ctx->in_ovoo.cap <= ctx->budget;
+  struct GiveBack {
+    tc_ctx *ctx;
+    ~GiveBack() {
+      if (ctx->ws_rns.cap > ctx->budget / 4) {
+        cudaDeviceSynchronize();                         // an early return may leave kernels in flight
+        ctx->ws_rns.release();
+      }
+    }
+  } give_back{ctx};
   if (rns) {
     const cudaError_t e = ctx->ws_rns.ensure(RL.total);
     if (e == cudaErrorMemoryAllocation) {

@@ -237,7 +237,11 @@ struct RnEnBatch {
   RnEnJob job[MAX_BATCH];
 };
 constexpr int RNS_GEMM_LAUNCHES = 2;       // storing, then adding
-constexpr int RNS_MIN_V = 8;
+// Smallest v of the residues: v = 8 is one whole DMMA tile but half an N = 16
+// chunk and half a 128-row tile here.  Whole calls, residues against DMMA: v = 8
+// o = 8 198 / 165 us, o = 16 538 / 438 us, o = 24 1056 / 1010 us; v = 9 o = 2
+// 105 / 113 us, o = 8 199 / 308 us, o = 16 536 / 1308 us.
+constexpr int RNS_MIN_V = 9;
 // Whether the path covers the shape (K bound of the exact FP32 sums).
 bool rns_supported(int o, int v);
 RnsGeom rns_geom(int o, int v);

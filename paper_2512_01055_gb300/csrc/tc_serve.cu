@@ -638,7 +638,8 @@ tc_status tc_submit(tc_ctx *ctx, const tc_job *job, uint64_t *ticket) {
               : tc::plan::make_dims(o, v, tc::fp64_tile());
   r->L = tc::plan::make_layout(r->d);
   if (split) r->SL = tc::split_layout(o, v, slices);
-  // FP64 on the tensor cores by the rule of the blocking entry points
+  // FP64 on the tensor cores as in the blocking entry points, within a quarter
+  // of the budget so that other jobs are admitted beside it
   if (!split && r->d.n_trip > 0 && tc::rns_supported(o, v)) {
     r->RL = tc::rns_layout(o, v, r->d.n_trip);
     if (r->RL.total <= ctx->budget / 4) r->group = tc::G_RNS;

@@ -160,3 +160,25 @@ def test_batched_jobs_of_different_widths_give_the_bits_of_each_alone():
         assert st.batched_jobs > st.iterations
     finally:
         tc.tc_finalize(ctx)
+
+
+# (4, 48) holds about 51 MB of images and W: no room for them; room, given back after the call; kept
+@pytest.mark.parametrize("budget_mb,kept", [(16, False), (128, False), (1024, True)])
+def test_images_within_the_budget_and_given_back(budget_mb, kept):
+    import torch
+    o, v = 4, 48
+    d = _random(o, v, 48)
+    e_ref, ref = _noalloc(o, v, d)
+    e_ijk = torch.zeros((o,) * 3, dtype=torch.float64, device="cuda")
+    ctx = tc.tc_init(0, hbm_budget_bytes=budget_mb << 20)
+    try:
+        args = (ctx, o, v, d["eps"], d["t1"], d["t2"], d["ovvv"], d["ovoo"], d["ovov"])
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        for _ in range(2):
+            r = tc.tc_energy_dev(*args, prec=tc.TC_FP64, e_ijk=e_ijk)
+            assert np.abs(e_ijk.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
+            assert abs(r.e_t - e_ref) <= TOL * np.abs(ref).sum()
+            assert (free - torch.cuda.mem_get_info()[0] > 32 << 20) == kept
+    finally:
+        tc.tc_finalize(ctx)
