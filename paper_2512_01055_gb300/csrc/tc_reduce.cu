@@ -24,6 +24,14 @@ __device__ __forceinline__ Comp combine(Comp a, const Comp &b) {
   return a;
 }
 
+// The lanes' sums combined by a fixed tree; lane 0 holds the result.
+__device__ __forceinline__ Comp warp_combine(Comp p) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+    p = combine(p, Comp{__shfl_down_sync(0xffffffffu, p.s, off), __shfl_down_sync(0xffffffffu, p.c, off)});
+  return p;
+}
+
 // One warp per triplet: lane q sums the item partials q, q + 32, ... in order,
 // the lanes are combined by a fixed tree.  Writes the weighted contribution and
 // leaves its (E, E[5]_ST) pair in the triplet's first partial slot.  One CTA
@@ -41,11 +49,8 @@ __global__ void __launch_bounds__(RT) reduce_triplets(const __grid_constant__ Re
       neumaier_add(p, x.x);
       neumaier_add(p5, x.y);
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      p = combine(p, Comp{__shfl_down_sync(0xffffffffu, p.s, off), __shfl_down_sync(0xffffffffu, p.c, off)});
-      p5 = combine(p5, Comp{__shfl_down_sync(0xffffffffu, p5.s, off), __shfl_down_sync(0xffffffffu, p5.c, off)});
-    }
+    p = warp_combine(p);
+    p5 = warp_combine(p5);
     __syncwarp();                                           // every lane's reads are done
     if (lane == 0) {
       const int4 tr = J.trip[t];
@@ -57,11 +62,17 @@ __global__ void __launch_bounds__(RT) reduce_triplets(const __grid_constant__ Re
   }
 }
 
-// One CTA per job: thread q sums triplets q, q + RT, ... in order, thread 0
-// combines the RT sums in thread order.
+// One CTA per job: thread q sums triplets q, q + RT, ... in order; the lanes of
+// a warp, then the warps, are combined by fixed trees.  Bound by the latency of
+// dependent FP64 additions: thread 0 adding up to RT sums in a row took about
+// 0.6 us a sum (whole split calls at o=6 v=36 182 us, with the trees 158 us; 0.11
+// to 0.23 ms less at o=13 v=131 and o=12 v=132).
 __global__ void __launch_bounds__(RT) reduce_jobs(const __grid_constant__ RedBatch B) {
   const RedJob &J = B.job[blockIdx.x];
-  __shared__ double ss[RT], sc[RT], sa[RT], s5[RT], c5[RT];
+  constexpr int NW = RT / 32;
+  __shared__ Comp s4[NW], s5[NW];
+  __shared__ double sa[NW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Comp a{0.0, 0.0}, a5{0.0, 0.0};
   double absum = 0.0;
   for (int t = threadIdx.x; t < J.n_trip; t += RT) {
@@ -70,22 +81,25 @@ __global__ void __launch_bounds__(RT) reduce_jobs(const __grid_constant__ RedBat
     neumaier_add(a5, x.y);
     absum += fabs(x.x);
   }
-  ss[threadIdx.x] = a.s;
-  sc[threadIdx.x] = a.c;
-  sa[threadIdx.x] = absum;
-  s5[threadIdx.x] = a5.s;
-  c5[threadIdx.x] = a5.c;
+  a = warp_combine(a);
+  a5 = warp_combine(a5);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) absum += __shfl_down_sync(0xffffffffu, absum, off);
+  if (lane == 0) { s4[warp] = a; s5[warp] = a5; sa[warp] = absum; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Comp tot{0.0, 0.0}, tot5{0.0, 0.0};
-    double ab = 0.0, cc = 0.0, cc5 = 0.0;
-    for (int i = 0; i < min(RT, J.n_trip); ++i) {
-      neumaier_add(tot, ss[i]); cc += sc[i]; ab += sa[i];
-      neumaier_add(tot5, s5[i]); cc5 += c5[i];
+  if (warp == 0) {
+    a = lane < NW ? s4[lane] : Comp{0.0, 0.0};
+    a5 = lane < NW ? s5[lane] : Comp{0.0, 0.0};
+    absum = lane < NW ? sa[lane] : 0.0;
+    a = warp_combine(a);
+    a5 = warp_combine(a5);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) absum += __shfl_down_sync(0xffffffffu, absum, off);
+    if (lane == 0) {
+      J.out[0] = a.s + a.c;
+      J.out[1] = absum;
+      J.out[2] = a5.s + a5.c;
     }
-    J.out[0] = tot.s + (tot.c + cc);
-    J.out[1] = ab;
-    J.out[2] = tot5.s + (tot5.c + cc5);
   }
 }
 
