@@ -6,11 +6,11 @@
 
 A step is one full (T) energy -- every hot-path stage: BF16 slicing into
 tensor-core images (split path), work tables, the W-term GEMM and orbit-energy
-kernels (split path; the FP64 path has one fused W/V/energy kernel), the
-compensated reduction and the read-back of E_T -- on one seeded synthetic job
-whose inputs are resident in HBM before timing starts.  The inputs (ovvv
-alone is 20.5 GB at o=40, v=400) exceed the 129 MB L2, so no L2 flush is
-needed between steps.
+kernels (FP64 path: residue images, residue GEMMs and energy kernel, or one
+fused W/V/energy kernel where those do not run), the compensated reduction and
+the read-back of E_T -- on one seeded synthetic job whose inputs are resident in
+HBM before timing starts.  The inputs (ovvv alone is 20.5 GB at o=40, v=400)
+exceed the 129 MB L2, so no L2 flush is needed between steps.
 
 Headline ("value"): the split-precision path (BF16 slices, s = --slices) on
 the precision workload o=40, v=400 (Q = 1320).  Beside it: one energy at each
@@ -122,7 +122,7 @@ class ClockSampler:
 def kernel_source_hash(prec):
     """Hash of the kernel source with comments and blank lines removed (a comment edit keeps it)."""
     import re
-    names = ["tc_fp64.cu"] if prec == "fp64" else ["tc_split.cu", "tc_ptx.cuh"]
+    names = ["tc_fp64.cu", "tc_rns.cu"] if prec == "fp64" else ["tc_split.cu", "tc_ptx.cuh"]
     paths = [os.path.join(ROOT, "paper_2512_01055_gb300", "csrc", n) for n in names]
     if not all(os.path.exists(p) for p in paths):
         return None
@@ -604,7 +604,13 @@ def main():
     # back to back for the whole energy, so the sustained (power-capped) peak applies.
     peak_bf16 = bf16_sus or bf16_peak
     which = "sustained" if bf16_sus else "burst"
-    if head_prec == tc.TC_FP64:
+    if head_prec == tc.TC_FP64 and head["wterm"] < head["kernel"]:
+        # FP64 in residues: 15 BF16 products per contraction, GEMM launches apart from the energy launches
+        kname, pairs = "rns_gemm_kernel", 15
+        peak = peak_bf16
+        peak_note = (f"BF16 dense {src} {which} peak; achieved counts the 15 residue products of the "
+                     f"2(o^3 v^4 + o^4 v^3) flop that form W (padding to tiles not counted)")
+    elif head_prec == tc.TC_FP64:
         kname, pairs = "tc_fp64_kernel", 1
         peak = peak_bf16 * FP64_NOMINAL_TF / BF16_NOMINAL_TF
         peak_note = f"FP64 tensor (DMMA) peak = {src} bf16 {which} x nominal FP64/BF16 ratio 1.25/2250"
@@ -621,7 +627,8 @@ def main():
                     "prep_ms": 1e3 * head["prep"], "kernels_ms": 1e3 * head["kernel"],
                     "wterm_ms": 1e3 * head["wterm"], "input_generation_s": t_gen})
         if head_prec == tc.TC_FP64:
-            dtype = "f64 (DMMA) throughout"
+            dtype = ("f64 accuracy: W as exact integer products in 15 bf16 residues; epilogue and sums f64"
+                     if kname == "rns_gemm_kernel" else "f64 (DMMA) throughout")
         else:
             dtype = (f"bf16x{head_slices} slices -> f32 tensor-core accumulation; epilogue (D, 1/D, quotients, "
                      f"sums over an item) in float pairs; per-triplet f64; compensated f64 total")
@@ -637,7 +644,7 @@ def main():
             "gpu_launches": head["launches"],
             "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak,
-                         "traffic": recorded_traffic(kname, name, "fp64" if pairs == 1 else "split"),
+                         "traffic": recorded_traffic(kname, name, "fp64" if head_prec == tc.TC_FP64 else "split"),
                          "kernel": kname, "kernel_ms": 1e3 * head["wterm"], "peak_source": peak_note},
         }
         out["df"] = df_line
@@ -650,12 +657,13 @@ def main():
                            "how": "tc_triplets_dev kernel time on the sampled triplets x all triplets / sampled"}
             out["config"]["speedup_split_vs_fp64"] = fp_s / head["sec"]
         if fp64 is not None:
-            fpeak = peak_bf16 * FP64_NOMINAL_TF / BF16_NOMINAL_TF
-            fach = flops / fp64["kernel"] / 1e12
+            rns = fp64["wterm"] < fp64["kernel"]             # FP64 in residues on the BF16 tensor cores
+            fpeak = peak_bf16 if rns else peak_bf16 * FP64_NOMINAL_TF / BF16_NOMINAL_TF
+            fach = flops * (15 if rns else 1) / fp64["wterm"] / 1e12
             out["fp64"] = {"value": world * flops / fp64["sec"] / 1e12, "unit": "TFLOP/s", "s_per_energy": fp64["sec"],
                            "steps": 1, "warmup": 1, "e_t": fp64["e_t"], "projected": False,
                            "roofline": {"bound": "tensor", "achieved": fach, "peak": fpeak, "frac": fach / fpeak,
-                                        "kernel": "tc_fp64_kernel"}}
+                                        "kernel": "rns_gemm_kernel" if rns else "tc_fp64_kernel"}}
             out["config"]["abs_dE_split_vs_fp64"] = abs(head["e_t"] - fp64["e_t"])
             out["config"]["rel_dE_split_vs_fp64"] = abs(head["e_t"] - fp64["e_t"]) / abs(fp64["e_t"])
             out["config"]["speedup_split_vs_fp64"] = fp64["sec"] / head["sec"]
