@@ -58,9 +58,17 @@ namespace tc {
 namespace {
 
 constexpr int RL = 15;                       // moduli
-// In pairs for the drain (the first of a pair at most 255, its residue packs
-// into a byte), the power of two last and alone.
-constexpr int MODULI[RL] = {255, 257, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 256};
+// In pairs for the drain, the power of two last and alone.  The first of a pair
+// packs its residue into a byte and is at most 253: with 255 the rounding of
+// c * fl(1/255) gives +128 for sums c from -8454907 down (K above 512, residues
+// of one sign), which a byte holds as -128.
+constexpr int MODULI[RL] = {253, 257, 251, 255, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 256};
+constexpr bool packed_fit() {
+  for (int l = 0; l + 1 < RL; l += 2)
+    if (MODULI[l] > 253) return false;
+  return true;
+}
+static_assert(packed_fit(), "the first modulus of a pair packs into a byte");
 constexpr int KMAX = 1024;                   // largest K whose residue products sum exactly in FP32
 // |sum of three F| <= 3 * 2^(BITS_A + BITS_B + 2) < P / 2 = 2^117.16
 constexpr int BITS_A = 57, BITS_B = 56;
