@@ -197,6 +197,8 @@ __device__ __forceinline__ int ilog2d(double x) {       // floor(log2 x) of a no
 //   [.., n1)  t2[r][q][z][:]      (o o v, length v)
 //   [.., n2)  ovoo[r][z][q][:]    (o v o, length o)
 //   then, one thread per column, t2[p][:][x][y] (o v v, length o)
+// A row whose squares all underflow gets the smallest denormal instead of the 0
+// of a row of zeros: an array of such rows is out of the grid's range.
 __global__ void rns_norms(Inputs in, int o, int v, Scales s) {
   const long long n0 = (long long)o * v * v, n1 = n0 + (long long)o * o * v, n2 = n1 + (long long)o * v * o;
   const int lane = threadIdx.x & 31;
@@ -208,9 +210,16 @@ __global__ void rns_norms(Inputs in, int o, int v, Scales s) {
     else if (w < n1) { src = in.t2 + (w - n0) * v; len = v; }
     else             { src = in.ovoo + (w - n1) * o; len = o; }
     double a = 0.0;
-    for (int k = lane; k < len; k += 32) a = fma(src[k], src[k], a);
+    bool any = false;
+    for (int k = lane; k < len; k += 32) {
+      const double t = src[k];
+      any |= t != 0.0;
+      a = fma(t, t, a);
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    any = __any_sync(0xffffffffu, any);
+    if (a == 0.0 && any) a = __longlong_as_double(1);
     if (lane == 0) {
       if (w < n0) {
         s.ra[w] = a;
@@ -229,11 +238,13 @@ __global__ void rns_norms(Inputs in, int o, int v, Scales s) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n0; e += (long long)gridDim.x * blockDim.x) {
     const long long p = e / vv, xy = e - p * vv;
     double a = 0.0;
+    bool any = false;
     for (int l = 0; l < o; ++l) {
       const double t = in.t2[(p * o + l) * vv + xy];
+      any |= t != 0.0;
       a = fma(t, t, a);
     }
-    s.rt[e] = a;
+    s.rt[e] = a == 0.0 && any ? __longlong_as_double(1) : a;
   }
 }
 

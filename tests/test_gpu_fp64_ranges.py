@@ -31,3 +31,17 @@ def test_long_sums_of_one_sign():
     print(f"max |de| / max |e| = {np.abs(e - ref).max() / scale:.2e}")
     assert np.abs(e - ref).max() <= 1e-12 * scale
     assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
+
+
+@pytest.mark.parametrize("what", ["t2", "ovvv and ovoo"])
+def test_norms_whose_squares_underflow(what):
+    """Operands at 2^-540: their squares are zero in FP64, their products with the other operands are not."""
+    o, v = 4, 21
+    d = _random(o, v, 93)
+    for n in what.split(" and "):
+        d[n] *= 2.0 ** -540
+    r, e = _energy(o, v, d)
+    e_ref, ref = _noalloc(o, v, d)
+    assert np.abs(ref).max() > 0.0
+    assert np.all(np.abs(e - ref) <= 1e-11 * np.abs(ref))
+    assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
