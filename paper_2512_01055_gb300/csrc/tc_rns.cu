@@ -24,11 +24,13 @@
 // right to about one unit in the last of 64 places.
 //
 // Scales.  W_ijk^abc is a sum of products with one fixed-point grid,
-// 2^-(e_a + e_b + e_c + u_i + u_j + u_k + SS): an exponent per virtual and per
-// occupied orbital from the norms of the integrals, and a global shift from
-// the norms of the scaled operands.  So the contributions of all six
-// permutations are integers on one grid: they are added by 64-bit integer
-// reductions in L2, which are exact and free of order.
+// 2^-(e_a + e_b + e_c + u_i + u_j + u_k + SS): an exponent >= 0 per virtual and
+// per occupied orbital from the norms of integrals and amplitudes together, and
+// a global shift from the largest norms.  The exponents raise no row above the
+// largest of its array, so they refine the grid of weak orbitals and coarsen
+// none.  The contributions of all six permutations are integers on one grid:
+// they are added by 64-bit integer reductions in L2, which are exact and free
+// of order.
 //
 // W as three GEMMs per triplet (F(p,q,r) of tc_split.cu, the same operand
 // segments):  W_abc = F(i,j,k)[ab,c] + F(i,k,j)[ac,b] + F(j,k,i)[bc,a].
@@ -176,20 +178,22 @@ constexpr double C_P = p_scaled();
 
 // ---------------------------------------------------------------- scales
 
-// Arrays of the scale search inside a job's scratch (all indexed by orbital):
-// squared norms of the operand rows, their maxima as IEEE bits, exponents.
+// Arrays of the scale search inside a job's scratch: squared norms of the
+// operand rows, their maxima per array and orbital as IEEE bits, exponents.
+// Arrays: 0 ovvv[p][x][y][:], 1 t2[p][:][x][y] (hole), 2 t2[r][q][z][:], 3 ovoo[r][z][q][:].
 struct Scales {
   double *ra, *rt, *rb, *rh;       // [o][v][v], [o][v][v], [o][o][v], [o][v][o]
-  unsigned long long *nv;          // [v]: largest squared row norm of ovvv with x at either place
-  unsigned long long *no;          // [o]: the same with p, after the virtual exponents
-  unsigned long long *mx;          // [4]: largest scaled squared norms of ovvv, t2 (hole), t2, ovoo rows
-  int *ev, *uo;                    // [v], [o] exponents
-  int *sh;                         // [5]: shifts of the four operands and SS
+  unsigned long long *nv, *no;     // [4][v], [4][o]: largest squared norm of the array's rows with that orbital
+  int *dv, *du;                    // [v], [o]: exponents that suit every array's largest rows, one orbital at a time
+  int *fv, *fu;                    // [v], [o]: share of them, in 256ths, that suits every row
+  int *ev, *uo;                    // [v], [o]: the exponents taken
+  int *sh;                         // [5]: shifts of the four operands and SS; sh[5]: 1 if any of dv, du is not 0
   int *flag;                       // 1: inputs out of the range the integer grid covers
 };
 
-__device__ __forceinline__ int ilog2d(double x) {       // floor(log2 x) of a normal positive x
-  return (int)((__double_as_longlong(x) >> 52) & 0x7FF) - 1023;
+// 0 for a zero of either sign.
+__device__ __forceinline__ unsigned magnitude(double x) {
+  return (unsigned)__double2hiint(x) << 1 | (unsigned)__double2loint(x);
 }
 
 // Squared norms of the operand rows, one warp per row:
@@ -197,12 +201,27 @@ __device__ __forceinline__ int ilog2d(double x) {       // floor(log2 x) of a no
 //   [.., n1)  t2[r][q][z][:]      (o o v, length v)
 //   [.., n2)  ovoo[r][z][q][:]    (o v o, length o)
 //   then, one thread per column, t2[p][:][x][y] (o v v, length o)
-// A row whose squares all underflow gets the smallest denormal instead of the 0
-// of a row of zeros: an array of such rows is out of the grid's range.
+// The maxima per orbital are collected in shared memory first (whole calls at
+// o=6 v=36 270 us; 283 us with a look at the global maxima for every row).  The
+// FP64 pipe bounds it at o=20 v=200, so zeros are told by their bits (FP64
+// comparisons: 0.5 ms more).  A row whose squares all underflow gets the smallest
+// denormal instead of the 0 of a row of zeros: an array of such rows is out of
+// the grid's range.
 __global__ void rns_norms(Inputs in, int o, int v, Scales s) {
   const long long n0 = (long long)o * v * v, n1 = n0 + (long long)o * o * v, n2 = n1 + (long long)o * v * o;
   const int lane = threadIdx.x & 31;
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+  extern __shared__ unsigned long long top[];              // [4][v] and [4][o], as s.nv and s.no
+  unsigned long long *const tv = top, *const to = top + 4 * v;
+  for (int x = threadIdx.x; x < 4 * (v + o); x += blockDim.x) top[x] = 0;
+  __syncthreads();
+  auto up = [](double a, unsigned long long *m0, unsigned long long *m1, unsigned long long *m2) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a);
+    unsigned long long *const m[3] = {m0, m1, m2};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)                            // most rows raise no maximum
+      if (b > *(volatile unsigned long long *)m[i]) atomicMax(m[i], b);
+  };
   for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < n2; w += warps) {
     const double *src;
     int len;
@@ -210,27 +229,29 @@ __global__ void rns_norms(Inputs in, int o, int v, Scales s) {
     else if (w < n1) { src = in.t2 + (w - n0) * v; len = v; }
     else             { src = in.ovoo + (w - n1) * o; len = o; }
     double a = 0.0;
-    bool any = false;
+    unsigned any = 0;                                      // by bits: a comparison would take the FP64 pipe, which bounds this
     for (int k = lane; k < len; k += 32) {
       const double t = src[k];
-      any |= t != 0.0;
+      any |= magnitude(t);
       a = fma(t, t, a);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-    any = __any_sync(0xffffffffu, any);
-    if (a == 0.0 && any) a = __longlong_as_double(1);
-    if (lane == 0) {
+    any = __any_sync(0xffffffffu, any != 0);
+    if (any && magnitude(a) == 0) a = __longlong_as_double(1);
+    if (lane == 0) {                                       // row numbers fit 32 bits (o, v <= 504)
       if (w < n0) {
+        const unsigned e = (unsigned)w;
         s.ra[w] = a;
-        const unsigned long long b = (unsigned long long)__double_as_longlong(a);
-        unsigned long long *nx = s.nv + (w / v) % v, *ny = s.nv + w % v;
-        if (b > *(volatile unsigned long long *)nx) atomicMax(nx, b);      // most rows raise no maximum
-        if (b > *(volatile unsigned long long *)ny) atomicMax(ny, b);
+        up(a, to + e / v / v, tv + e / v % v, tv + e % v);
       } else if (w < n1) {
-        s.rb[w - n0] = a;
+        const unsigned e = (unsigned)(w - n0);
+        s.rb[e] = a;
+        up(a, to + 2 * o + e / v / o, to + 2 * o + e / v % o, tv + 2 * v + e % v);
       } else {
-        s.rh[w - n1] = a;
+        const unsigned e = (unsigned)(w - n1);
+        s.rh[e] = a;
+        up(a, to + 3 * o + e / o / v, to + 3 * o + e % o, tv + 3 * v + e / o % v);
       }
     }
   }
@@ -238,101 +259,125 @@ __global__ void rns_norms(Inputs in, int o, int v, Scales s) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n0; e += (long long)gridDim.x * blockDim.x) {
     const long long p = e / vv, xy = e - p * vv;
     double a = 0.0;
-    bool any = false;
+    unsigned any = 0;
     for (int l = 0; l < o; ++l) {
       const double t = in.t2[(p * o + l) * vv + xy];
-      any |= t != 0.0;
+      any |= magnitude(t);
       a = fma(t, t, a);
     }
-    s.rt[e] = a == 0.0 && any ? __longlong_as_double(1) : a;
+    if (any && magnitude(a) == 0) a = __longlong_as_double(1);
+    s.rt[e] = a;
+    up(a, to + o + p, tv + v + (unsigned)xy / v, tv + v + (unsigned)xy % v);
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < 4 * (v + o); x += blockDim.x) {
+    unsigned long long *const m = x < 4 * v ? s.nv + x : s.no + (x - 4 * v);
+    if (top[x] > *(volatile unsigned long long *)m) atomicMax(m, top[x]);
   }
 }
 
-// Exponent of an orbital: the squared norm n2 brought next to the largest one
-// (powers of two, from exponents alone: scaling an input array by a power of
-// two changes none of them).
-__device__ __forceinline__ int rel_exp(unsigned long long bits, int emax) {
-  if (bits == 0) return 0;
-  const int e = ilog2d(__longlong_as_double((long long)bits));
-  return min(max((emax - e) / 2, 0), 40);
+// Exponents.  A row of array k may be scaled up by its slack, the powers of two
+// between its norm and the array's largest (from binary exponents alone, so
+// scaling an input array by a power of two changes none of them).  d of an
+// orbital is the least slack of the rows that hold it, over all four arrays: 0
+// where any array has a row of full size.  A row holds three orbitals, so the
+// sum of their d may exceed its slack; each orbital then takes the share
+// slack / sum of its d, the smallest over its rows, which keeps every row
+// within the array's largest.  (Where all arrays carry one factor per orbital,
+// the shares stay near 1 and the exponents take it out.  An exponent from the
+// integrals alone, used before, scaled amplitudes up with it: W lost all digits
+// when one orbital's ovvv was 2^-24 of the others'.)
+constexpr int D_MAX = 16;
+constexpr int NO_ROW = 1 << 20;                           // slack of a row of zeros
+
+// Slack of a squared norm (IEEE bits) against the array's largest.
+__device__ __forceinline__ int slack(unsigned long long bits, int emax) {
+  return bits == 0 ? NO_ROW : max(emax - ((int)(bits >> 52) - 1023), 0) / 2;
+}
+__device__ __forceinline__ int expo(unsigned long long bits) { return (int)(bits >> 52) - 1023; }
+
+// Each array's largest squared norm (IEEE bits), to every thread of the CTA.
+__device__ void array_max(int v, const Scales &s, unsigned long long (&mb)[4]) {
+  __shared__ unsigned long long m[4];
+  if (threadIdx.x < 4) m[threadIdx.x] = 0;
+  __syncthreads();
+  for (int k = 0; k < 4; ++k)
+    for (int x = threadIdx.x; x < v; x += blockDim.x) {
+      const unsigned long long b = __ldcg(s.nv + (size_t)k * v + x);
+      if (b > *(volatile unsigned long long *)(m + k)) atomicMax(m + k, b);
+    }
+  __syncthreads();
+  for (int k = 0; k < 4; ++k) mb[k] = m[k];
+  __syncthreads();
 }
 
-// Virtual exponents, by one CTA.
-__device__ void virtual_exps(int v, const Scales &s) {
-  __shared__ unsigned long long m;
-  if (threadIdx.x == 0) m = 0;
+// d of every orbital, shares of 256 / 256, by one CTA.
+__device__ void wanted(int o, int v, const Scales &s) {
+  unsigned long long mb[4];
+  array_max(v, s, mb);
+  if (threadIdx.x == 0) s.sh[5] = 0;
   __syncthreads();
-  for (int x = threadIdx.x; x < v; x += blockDim.x) atomicMax(&m, s.nv[x]);
-  __syncthreads();
-  const int emax = m ? ilog2d(__longlong_as_double((long long)m)) : 0;
-  for (int x = threadIdx.x; x < v; x += blockDim.x) s.ev[x] = rel_exp(s.nv[x], emax);
-}
-
-// 4^e as a double (|e| <= 500)
-__device__ __forceinline__ double pow4(int e) { return __longlong_as_double((long long)(1023 + 2 * e) << 52); }
-
-// Largest row norm of occupied orbital p after the virtual exponents.
-__device__ void occ_norms(int p, int v, const Scales &s) {
-  const long long vv = (long long)v * v;
-  unsigned long long b = 0;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < vv; e += (long long)gridDim.x * blockDim.x) {
-    const double a = s.ra[p * vv + e] * pow4(s.ev[e / v] + s.ev[e % v]);
-    b = max(b, (unsigned long long)__double_as_longlong(a));
+  for (int x = threadIdx.x; x < v + o; x += blockDim.x) {
+    const bool vir = x < v;
+    int d = NO_ROW;
+    for (int k = 0; k < 4; ++k)
+      d = min(d, slack(__ldcg(vir ? s.nv + (size_t)k * v + x : s.no + (size_t)k * o + (x - v)), expo(mb[k])));
+    d = d == NO_ROW ? 0 : min(d, D_MAX);
+    (vir ? s.dv[x] : s.du[x - v]) = d;
+    (vir ? s.fv[x] : s.fu[x - v]) = 256;
+    if (d) s.sh[5] = 1;
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(s.no + p, b);
 }
 
-__device__ __forceinline__ int occ_exp(const Scales &s, int o, int p) {
-  unsigned long long m = 0;
-  for (int q = 0; q < o; ++q) m = max(m, __ldcg(s.no + q));
-  return rel_exp(__ldcg(s.no + p), m ? ilog2d(__longlong_as_double((long long)m)) : 0);
-}
-
-// Largest scaled squared norms of the four operands.
-__device__ void max_norms(int o, int v, const Scales &s, int *uo) {
-  for (int p = threadIdx.x; p < o; p += blockDim.x) {
-    uo[p] = occ_exp(s, o, p);
-    if (blockIdx.x == 0) s.uo[p] = uo[p];
-  }
-  __syncthreads();
+// Shares: every row's slack against the sum of its orbitals' d.
+__device__ void shares(int o, int v, const Scales &s) {
+  if (__ldcg(s.sh + 5) == 0) return;
+  unsigned long long mb[4];
+  array_max(v, s, mb);
   const long long vv = (long long)v * v, n0 = (long long)o * vv, n1 = (long long)o * o * v;
-  unsigned long long b[4] = {0, 0, 0, 0};
-  auto up = [](unsigned long long &m, double a) { m = max(m, (unsigned long long)__double_as_longlong(a)); };
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, st = (long long)gridDim.x * blockDim.x;
+  auto row = [&](double n, int k, const int *d0, const int *d1, const int *d2, int *f0, int *f1, int *f2) {
+    const int sum = __ldcg(d0) + __ldcg(d1) + __ldcg(d2);
+    const int sl = slack((unsigned long long)__double_as_longlong(n), expo(mb[k]));
+    if (sl >= sum) return;
+    const int f = 256 * sl / sum;
+    int *const ff[3] = {f0, f1, f2};
+    for (int i = 0; i < 3; ++i)
+      if (f < *(volatile int *)ff[i]) atomicMin(ff[i], f);
+  };
   for (long long e = t; e < n0; e += st) {
-    const long long p = e / vv, xy = e - p * vv;
-    const double f = pow4(s.ev[xy / v] + s.ev[xy % v] + uo[p]);
-    up(b[0], s.ra[e] * f);
-    up(b[1], s.rt[e] * f);
+    const int p = (int)(e / vv), x = (int)(e % vv / v), y = (int)(e % v);
+    row(s.ra[e], 0, s.du + p, s.dv + x, s.dv + y, s.fu + p, s.fv + x, s.fv + y);
+    row(s.rt[e], 1, s.du + p, s.dv + x, s.dv + y, s.fu + p, s.fv + x, s.fv + y);
   }
   for (long long e = t; e < n1; e += st) {
     const int z = (int)(e % v), q = (int)(e / v % o), r = (int)(e / v / o);
-    up(b[2], s.rb[e] * pow4(s.ev[z] + uo[r] + uo[q]));
+    row(s.rb[e], 2, s.du + r, s.du + q, s.dv + z, s.fu + r, s.fu + q, s.fv + z);
     const int q2 = (int)(e % o), z2 = (int)(e / o % v), r2 = (int)(e / o / v);
-    up(b[3], s.rh[e] * pow4(s.ev[z2] + uo[r2] + uo[q2]));
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) b[k] = max(b[k], __shfl_xor_sync(0xffffffffu, b[k], off));
-    if ((threadIdx.x & 31) == 0) atomicMax(s.mx + k, b[k]);
+    row(s.rh[e], 3, s.du + r2, s.du + q2, s.dv + z2, s.fu + r2, s.fu + q2, s.fv + z2);
   }
 }
 
-// Shifts of the four operands (one thread).  A row of norm n is scaled to at
+// The exponents taken.
+__device__ void take_exps(int o, int v, const Scales &s) {
+  for (int x = threadIdx.x; x < v; x += blockDim.x) s.ev[x] = s.dv[x] * __ldcg(s.fv + x) >> 8;
+  for (int p = threadIdx.x; p < o; p += blockDim.x) s.uo[p] = s.du[p] * __ldcg(s.fu + p) >> 8;
+}
+
+// Shifts of the four operands (one CTA).  A row of norm n is scaled to at
 // most 2^BITS: i = ceil(log2 of the largest norm).  Particle and hole products
 // share the grid (sa + sb = sah + sbh = SS); the pair with room to spare is
 // scaled down.  Arrays of zeros take shift 0; inputs whose norms leave
 // [2^-100, 2^100] or are not finite set the flag.
-__device__ void shifts(const Scales &s) {
+__device__ void shifts(int v, const Scales &s) {
+  unsigned long long mb[4];
   int i[4];
   bool any[4];
+  array_max(v, s, mb);
+  if (threadIdx.x != 0) return;
   for (int k = 0; k < 4; ++k) {
-    const unsigned long long b = __ldcg(s.mx + k);
-    any[k] = b != 0;
-    const int e = any[k] ? (int)(b >> 52) - 1023 : 0;
+    any[k] = mb[k] != 0;
+    const int e = any[k] ? expo(mb[k]) : 0;
     if (any[k] && (e < -200 || e > 200)) *s.flag = 1;
     i[k] = (e + 202) / 2 - 100;                    // ceil((e + 1) / 2)
   }
@@ -355,26 +400,23 @@ __device__ void shifts(const Scales &s) {
   s.sh[4] = sa + sb;
 }
 
-__global__ void rns_virtual_exps(int v, Scales s) { virtual_exps(v, s); }
-__global__ void rns_occ_norms(int v, Scales s) { occ_norms(blockIdx.y, v, s); }
-__global__ void rns_max_norms(int o, int v, Scales s) {
-  extern __shared__ int uo[];
-  max_norms(o, v, s, uo);
+__global__ void rns_wanted(int o, int v, Scales s) { wanted(o, v, s); }
+__global__ void rns_shares(int o, int v, Scales s) { shares(o, v, s); }
+__global__ void rns_scales(int o, int v, Scales s) {
+  take_exps(o, v, s);
+  shifts(v, s);
 }
-__global__ void rns_shifts(Scales s) { shifts(s); }
 
-// All four steps by one CTA, for jobs where their launches take longer than
+// All three steps by one CTA, for jobs where their launches take longer than
 // their work: up to SCALES_ONE rows of ovvv.
 constexpr long long SCALES_ONE = 1 << 16;
 __global__ void __launch_bounds__(1024) rns_scales_one(int o, int v, Scales s) {
-  extern __shared__ int uo[];
-  virtual_exps(v, s);
+  wanted(o, v, s);
   __syncthreads();
-  for (int p = 0; p < o; ++p) occ_norms(p, v, s);
+  shares(o, v, s);
   __syncthreads();
-  max_norms(o, v, s, uo);
-  __syncthreads();
-  if (threadIdx.x == 0) shifts(s);
+  take_exps(o, v, s);
+  shifts(v, s);
 }
 
 // ---------------------------------------------------------------- operand images
@@ -1236,12 +1278,16 @@ Scales scales_at(const RnsLayout &L, void *ws, int *flag) {
   s.rt = (double *)(b + L.rt);
   s.rb = (double *)(b + L.rb);
   s.rh = (double *)(b + L.rh);
+  const int v = L.g.v, o = L.g.o;
   s.nv = (unsigned long long *)(b + L.mx);
-  s.no = s.nv + L.g.v;
-  s.mx = s.no + L.g.o;
+  s.no = s.nv + 4 * v;
   s.ev = (int *)(b + L.ex);
-  s.uo = s.ev + L.g.v;
-  s.sh = s.uo + L.g.o;
+  s.uo = s.ev + v;
+  s.dv = s.uo + o;
+  s.du = s.dv + v;
+  s.fv = s.du + o;
+  s.fu = s.fv + v;
+  s.sh = s.fu + o;
   s.flag = flag;
   return s;
 }
@@ -1351,8 +1397,8 @@ RnsLayout rns_layout(int o, int v, int n_trip) {
   L.rt = take(O * V * V * 8);
   L.rb = take(O * O * V * 8);
   L.rh = take(O * V * O * 8);
-  L.mx = take((V + O + 4) * 8);
-  L.ex = take((V + O + 8) * 4);
+  L.mx = take(4 * (V + O) * 8);
+  L.ex = take((3 * (V + O) + 8) * 4);
   L.unit = take((size_t)3 * std::max(1, n_trip) * 4);
   L.need = take(O * O);
   L.total = off;
@@ -1379,7 +1425,7 @@ RnsTables rns_tables(int o, const int4 *trip, int n) {
   return t;
 }
 
-int rns_prep_launches(int o, int v) { return (long long)o * v * v <= SCALES_ONE ? 3 : 6; }
+int rns_prep_launches(int o, int v) { return (long long)o * v * v <= SCALES_ONE ? 3 : 5; }
 
 cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, const RnsTables &t, bool all, int *flag,
                             cudaStream_t st) {
@@ -1388,17 +1434,16 @@ cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, cons
   const Scales s = scales_at(L, ws, flag);
   cudaError_t e = cudaMemcpyAsync(b + L.unit, t.unit.data(), t.unit.size() * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !all) e = cudaMemcpyAsync(b + L.need, t.need.data(), t.need.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b + L.mx, 0, ((size_t)g.v + g.o + 4) * 8, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b + L.mx, 0, 4 * ((size_t)g.v + g.o) * 8, st);
   if (e != cudaSuccess) return e;
   const unsigned char *need = all ? nullptr : (const unsigned char *)(b + L.need);
-  rns_norms<<<PREP_BLOCKS, PREP_THREADS, 0, st>>>(in, g.o, g.v, s);
+  rns_norms<<<PREP_BLOCKS, PREP_THREADS, 4 * ((size_t)g.v + g.o) * 8, st>>>(in, g.o, g.v, s);
   if ((long long)g.o * g.v * g.v <= SCALES_ONE) {
-    rns_scales_one<<<1, 1024, (size_t)g.o * sizeof(int), st>>>(g.o, g.v, s);
+    rns_scales_one<<<1, 1024, 0, st>>>(g.o, g.v, s);
   } else {
-    rns_virtual_exps<<<1, 512, 0, st>>>(g.v, s);
-    rns_occ_norms<<<dim3(16, g.o), 256, 0, st>>>(g.v, s);
-    rns_max_norms<<<152 * 2, 256, (size_t)g.o * sizeof(int), st>>>(g.o, g.v, s);
-    rns_shifts<<<1, 1, 0, st>>>(s);
+    rns_wanted<<<1, 512, 0, st>>>(g.o, g.v, s);
+    rns_shares<<<152 * 2, 256, 0, st>>>(g.o, g.v, s);
+    rns_scales<<<1, 512, 0, st>>>(g.o, g.v, s);
   }
   unsigned char *ub = (unsigned char *)b;
   const long long work = (long long)g.o * ((g.v + 7) / 8) * ((g.v + 3) / 4) * g.hv;   // warps of the largest task

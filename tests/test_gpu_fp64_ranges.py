@@ -45,3 +45,56 @@ def test_norms_whose_squares_underflow(what):
     assert np.abs(ref).max() > 0.0
     assert np.all(np.abs(e - ref) <= 1e-11 * np.abs(ref))
     assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
+
+
+def _scale(d, what, k):
+    """d with the named operands of one occupied or one virtual orbital (or a block of pairs) times 2^-k."""
+    import torch
+    o, v = d["t1"].shape
+    d = {n: x.clone() for n, x in d.items()}
+    f, p, x = 2.0 ** -k, 2, 5
+    ints = what.startswith("ints")
+    if what == "t2_fragments":                      # pairs between {0, 1} and the rest, and two virtual blocks
+        d["t2"][:2, 2:] *= f
+        d["t2"][2:, :2] *= f
+        d["t2"][:, :, :9, 9:] *= f
+        d["t2"][:, :, 9:, :9] *= f
+        return d
+    if what in ("ovvv_occ", "ints_occ"):
+        d["ovvv"][p] *= f
+    if what in ("ovvv_vir", "ints_vir"):
+        for a in range(1, 4):
+            d["ovvv"].select(a, x).mul_(f)
+    if what in ("ovoo_occ", "ints_occ"):
+        for a in (0, 2, 3):
+            d["ovoo"].select(a, p).mul_(f)
+    if what in ("ovoo_vir", "ints_vir"):
+        d["ovoo"][:, x] *= f
+    if ints:
+        axes = (0, 2) if what == "ints_occ" else (1, 3)
+        for a in axes:
+            d["ovov"].select(a, p if what == "ints_occ" else x).mul_(f)
+    if what == "t2_occ":
+        for a in (0, 1):
+            d["t2"].select(a, p).mul_(f)
+    if what == "t2_vir":
+        for a in (2, 3):
+            d["t2"].select(a, x).mul_(f)
+    return d
+
+
+WHAT = ["ovvv_occ", "ovvv_vir", "ovoo_occ", "ovoo_vir", "t2_occ", "t2_vir", "ints_occ", "ints_vir"]
+
+
+@pytest.mark.parametrize("what", WHAT)
+@pytest.mark.parametrize("k", [8, 16, 24, 32, 40])
+def test_operands_of_one_orbital_smaller_than_the_others(what, k):
+    o, v = 5, 24
+    d = _scale(_random(o, v, 611), what, k)
+    r, e = _energy(o, v, d)
+    assert r.prep_seconds > 0.0 and r.wterm_seconds < r.kernel_seconds
+    e_ref, ref = _noalloc(o, v, d)
+    scale = np.abs(ref).max()
+    print(f"{what} 2^-{k}: max |de| / max |e| = {np.abs(e - ref).max() / scale:.2e}, dE/E = {abs(r.e_t / e_ref - 1):.2e}")
+    assert np.abs(e - ref).max() <= 1e-12 * scale
+    assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
