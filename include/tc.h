@@ -58,11 +58,13 @@ typedef enum {
 
 typedef enum {
   TC_FP64 = 0,         /* FP64-accurate W, FP64 epilogue and sums.  W as exact integer products in residues on
-                          the BF16 tensor cores: operands rounded once to a common power-of-two grid at least 2^-53
-                          of their norms, W to 64 bits (an error below that of FP64 accumulation); or with FP64
-                          tensor-core (DMMA) tiles where the shape (o < 2, v < 9, K = 2v + 2o padded above 1024),
-                          the memory (budget and device) or the inputs (infinities, NaN, norms outside 2^+-100)
-                          do not allow it */
+                          the BF16 tensor cores: operands rounded once to one power-of-two grid per array (refined
+                          for orbitals that are weak in every array), W to 64 bits.  W of a triplet is within about
+                          2^-50 of its root mean square, as FP64 accumulation leaves it; triplets too weak for that
+                          on the common grid are formed again with FP64 tensor-core (DMMA) tiles.  Everything runs
+                          on DMMA tiles where the shape (o < 2, v < 9, K = 2v + 2o padded above 1024), the memory
+                          (budget and device) or the inputs (infinities, NaN, an array's largest norm outside
+                          2^+-100) do not allow residues; the two agree to the accuracy stated, not to the bit */
   TC_SPLIT_BF16 = 1    /* W built from BF16 slices on tcgen05 tensor cores, FP32 accumulation;
                           V and the Eq. 1 bracket in FP32; D, 1/D, each point's quotient and
                           the sums over a work item in float pairs (~48 significant bits);

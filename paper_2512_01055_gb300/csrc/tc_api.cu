@@ -98,7 +98,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   // 0.8 s (4.3 ps a byte) to the 50 s of o=40 v=400, and the DMMA kernel does
   // 0.9 flop per ps, so 12 v^4 flop a triplet against 10 flop a byte leaves a
   // factor of 2.5 (the whole energy: 71 against 1.0 TFLOP/s).
-  const tc::RnsLayout RL = split ? tc::RnsLayout{} : tc::rns_layout(o, v, d.n_trip);
+  const tc::RnsLayout RL = split ? tc::RnsLayout{} : tc::rns_layout(d);
   bool rns = !split && !dmma && d.n_trip > 0 && tc::rns_supported(o, v) &&
              (RL.total <= ctx->budget / 4 || 12.0 * d.n_trip * v * v * v * v >= 10.0 * RL.total) &&
              need + RL.total + ctx->in_ovvv.cap + ctx->in_t2.cap + ctx->in_ovov.cap + ctx->in_ovoo.cap <= ctx->budget;
@@ -241,23 +241,44 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
     const tc_status ss = stage_upto(o);
     if (ss != TC_OK) return ss;
   }
-  {
-    tc::RedBatch rb{};
-    rb.njobs = 1;
-    rb.job[0] = tc::RedJob{d.n_trip, d.items_per_trip, o, w.trip, w.partial, e_trip, e_ijk_dev, dout};
-    TC_CUDA(ctx, tc::launch_reduce(rb, st));
-  }
-  TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out, dout, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-  TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out + 3, w.err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+  tc::RedBatch rb{};
+  rb.njobs = 1;
+  rb.job[0] = tc::RedJob{d.n_trip, d.items_per_trip, o, w.trip, w.partial, e_trip, e_ijk_dev, dout};
+  if (rns) tc::rns_weak(RL, ctx->ws_rns.p, &rb.job[0]);
+  TC_CUDA(ctx, tc::launch_reduce(rb, st));
+  TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out, dout, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
+  TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out + 4, w.err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   TC_CUDA(ctx, cudaStreamSynchronize(st));
   int errs[2] = {0, 0};
-  std::memcpy(errs, ctx->host_out + 3, sizeof errs);
+  std::memcpy(errs, ctx->host_out + 4, sizeof errs);
   const int errflag = errs[0];
   if (errflag != 0)
     return fail(ctx, (errflag >= 11 && errflag <= 15) ? TC_ETIMEOUT : TC_EINTERNAL,
                 "device-side wait gave up (code %d)", errflag);
   // inputs beyond the integer grid's range (infinities, NaN, norms outside 2^+-100): the DMMA kernel
   if (rns && errs[1] != 0) return run_device(ctx, o, v, in, prec, slices, e_ijk_dev, st, out, subset, e_sub, stg, true);
+  const int nweak = rns ? (int)ctx->host_out[3] : 0;
+  if (nweak > 0) {
+    // triplets too weak for the common grid: again by the DMMA kernel, into the same partials
+    tc::RedJob &J = rb.job[0];
+    J.list = J.weak;
+    J.nlist = nweak;
+    J.margin = nullptr;
+    int per_sm = 0;
+    TC_CUDA(ctx, tc::fp64_blocks_per_sm(&per_sm));
+    tc::FpBatch b{};
+    b.njobs = 1;
+    b.total_items = (long long)nweak * d.items_per_trip;
+    b.counter = w.counter;
+    b.job[0] = tc::FpJob{d, in, w, 0, 0, J.list};
+    TC_CUDA(ctx, cudaEventRecord(ctx->ev[4], st));
+    TC_CUDA(ctx, tc::launch_fp64(b, (int)std::min<long long>((long long)ctx->num_sms * per_sm, b.total_items), st));
+    TC_CUDA(ctx, cudaEventRecord(ctx->ev[5], st));
+    TC_CUDA(ctx, tc::launch_reduce(rb, st));
+    TC_CUDA(ctx, cudaMemcpyAsync(ctx->host_out, dout, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    TC_CUDA(ctx, cudaStreamSynchronize(st));
+    launches += 3;
+  }
   out->e_t = ctx->host_out[0];
   out->e_t5 = ctx->host_out[2];
   if (e_sub) {
@@ -279,6 +300,11 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
         wsum += 1e-3 * ms;
       }
       out->wterm_seconds = wsum;
+    }
+    if (nweak > 0) {
+      TC_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]));
+      out->kernel_seconds += 1e-3 * ms;
+      out->wterm_seconds += 1e-3 * ms;
     }
   }
   if (split && stg) {
@@ -395,9 +421,10 @@ tc_status tc_init(tc_ctx **out, const tc_options *opt) {
       cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
       cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaMallocHost((void **)&ctx->host_out, 4 * sizeof(double)) != cudaSuccess ||
+      cudaMallocHost((void **)&ctx->host_out, 6 * sizeof(double)) != cudaSuccess ||
       cudaEventCreate(&ctx->ev[0]) != cudaSuccess || cudaEventCreate(&ctx->ev[1]) != cudaSuccess ||
-      cudaEventCreate(&ctx->ev[2]) != cudaSuccess || cudaEventCreate(&ctx->ev[3]) != cudaSuccess) {
+      cudaEventCreate(&ctx->ev[2]) != cudaSuccess || cudaEventCreate(&ctx->ev[3]) != cudaSuccess ||
+      cudaEventCreate(&ctx->ev[4]) != cudaSuccess || cudaEventCreate(&ctx->ev[5]) != cudaSuccess) {
     delete ctx;
     return TC_ECUDA;
   }

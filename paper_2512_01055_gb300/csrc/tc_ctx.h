@@ -51,7 +51,7 @@ struct tc_ctx {
   tc::DevBuf df_in;                         // tc_energy_df: the device copy of B
   cudaEvent_t dfev[2] = {nullptr, nullptr}; // around the integral assembly
   double *host_out = nullptr;               // pinned read-back slot
-  cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};     // kernel timing
+  cudaEvent_t ev[6] = {};                   // kernel timing: kernels, preparation, weak triplets of the FP64 path
   std::vector<cudaEvent_t> wev;             // split path: a pair around each W-term launch (grown on demand)
   cudaStream_t copy_stream = nullptr;       // tc_energy: host-to-device copies of the inputs, by occupied-index chunk
   std::vector<cudaEvent_t> cev;             // tc_energy: one per chunk, recorded on copy_stream after its copies

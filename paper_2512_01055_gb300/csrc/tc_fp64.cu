@@ -63,8 +63,9 @@ tc_fp64_kernel(const __grid_constant__ FpBatch B) {
     const long long item = gitem - B.job[jc].item0 + B.job[jc].item_base;
     const int o = d.o, v = d.v;
     const long long vv = (long long)v * v;
-    const int t = (int)(item / d.items_per_trip);
+    int t = (int)(item / d.items_per_trip);
     const int chunk = (int)(item % d.items_per_trip);
+    if (B.job[jc].list) t = B.job[jc].list[t];
     const int4 tr = w.trip[t];
     const int occ[3] = {tr.x, tr.y, tr.z};
     double acc = 0.0, acc5 = 0.0;                // E_(T) and its V part E[5]_ST
@@ -210,8 +211,9 @@ tc_fp64_kernel(const __grid_constant__ FpBatch B) {
     if (tid == 0) {
       double s = 0.0, s5 = 0.0;
       for (int i2 = 0; i2 < THREADS / 32; ++i2) { s += s_red[i2]; s5 += s_red5[i2]; }
-      w.partial[2 * item] = s;
-      w.partial[2 * item + 1] = s5;
+      const long long slot = (long long)t * d.items_per_trip + chunk;
+      w.partial[2 * slot] = s;
+      w.partial[2 * slot + 1] = s5;
     }
     __syncthreads();
   }

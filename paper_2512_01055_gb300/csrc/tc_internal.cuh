@@ -69,6 +69,7 @@ struct FpJob {
   Work w;
   long long item0;     // first global item of this job in the launch
   long long item_base; // the job's own index of that item (a launch may run a slice of a job)
+  const int *list;     // optional: the job's items are those of these triplets (their partials' places unchanged)
 };
 struct FpBatch {
   int njobs;
@@ -188,10 +189,11 @@ struct RnsGeom {
   int nb;                // triplets per block (capacity of the W buffer)
 };
 // Byte offsets inside a job's workspace: operand images, W buffer, the scale
-// search's norms, maxima and exponents, unit table, mask of occupied pairs.
+// search's norms, maxima and exponents, unit table, the items' margins over
+// the weak triplets' bound and the list of weak triplets, mask of occupied pairs.
 struct RnsLayout {
   RnsGeom g;
-  size_t pa, pa2, hc, hc2, tb, hb, y, ra, rt, rb, rh, mx, ex, unit, need;
+  size_t pa, pa2, hc, hc2, tb, hb, y, ra, rt, rb, rh, mx, ex, unit, margin, weak, need;
   size_t total;
 };
 // Host tables of a triplet list.  A unit is one F GEMM of one triplet:
@@ -228,6 +230,7 @@ struct RnEnJob {         // one job's block of triplets in an energy launch
   const long long *y;
   const int *ev, *uo, *sh;
   double *partial;       // [n_items][2], slot t * items_per_trip + chunk
+  double *margin;        // [n_items]: |E[4]_ST| of the item less the weak triplets' bound
   int t0, nt;
   long long item0;
 };
@@ -245,7 +248,7 @@ constexpr int RNS_MIN_V = 9;
 // Whether the path covers the shape (K bound of the exact FP32 sums).
 bool rns_supported(int o, int v);
 RnsGeom rns_geom(int o, int v);
-RnsLayout rns_layout(int o, int v, int n_trip);
+RnsLayout rns_layout(const Dims &d);
 RnsTables rns_tables(int o, const int4 *trip, int n);
 // Scales, operand images and unit table (all: every occupied pair's images,
 // else those t.need marks).  *flag (device) is set to 1 when the inputs leave
@@ -262,6 +265,12 @@ cudaError_t launch_rns_block(RnBatch *gb, RnEnBatch &eb, int num_sms, cudaStream
 // As split_block_params: gp[0], gp[1], ep must run in this order.
 cudaError_t rns_block_params(RnBatch *gb, RnEnBatch &eb, int num_sms, void **gargs, void **eargs,
                              cudaKernelNodeParams *gp, cudaKernelNodeParams *ep);
+
+// Fill in the fields by which the reduction lists the weak triplets: those whose
+// W lies too far below the common grid's range.  The caller forms them again with
+// the DMMA kernel (FpJob::list) and reduces them a second time (RedJob::list).
+struct RedJob;
+void rns_weak(const RnsLayout &L, void *ws, RedJob *j);
 
 // ---------------------------------------------------------------- integrals from DF factors (tc_df.cu)
 // (ia|bd), (ia|jl) and (ia|jb) from B[nq][o+v][o+v] (Eq. 6) as exact digit
@@ -281,7 +290,11 @@ struct RedJob {
   double *partial;       // [n_trip][items_per_trip][2]; each triplet's first pair is overwritten by its sums
   double *e_trip;        // [n_trip] weighted triplet contributions
   double *e_ijk;         // optional [o][o][o]
-  double *out;           // [3]: E, sum |e| and E[5]_ST
+  double *out;           // [4]: E, sum |e|, E[5]_ST and the number of weak triplets
+  const double *margin;  // optional [n_trip][items_per_trip]: a triplet of negative (or NaN) sum is weak
+  int *weak_n, *weak;    // with margin: their number (zero before) and their indices, in any order
+  const int *list;       // optional: only the partials of these nlist triplets are new; the others' are their sums
+  int nlist;
 };
 struct RedBatch {
   int njobs;

@@ -34,23 +34,33 @@ __device__ __forceinline__ Comp warp_combine(Comp p) {
 
 // One warp per triplet: lane q sums the item partials q, q + 32, ... in order,
 // the lanes are combined by a fixed tree.  Writes the weighted contribution and
-// leaves its (E, E[5]_ST) pair in the triplet's first partial slot.  One CTA
+// leaves its (E, E[5]_ST) pair in the triplet's first partial slot, and lists
+// the triplet where its margin is negative.  One CTA
 // with a thread per triplet did this before: 1.6 ms of FP64 latency at o=12
 // v=132 (352 triplets of 969 items).
 __global__ void __launch_bounds__(RT) reduce_triplets(const __grid_constant__ RedBatch B) {
   const RedJob &J = B.job[blockIdx.y];
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (RT / 32);
-  for (int t = blockIdx.x * (RT / 32) + (threadIdx.x >> 5); t < J.n_trip; t += nw) {
+  const int n = J.list ? J.nlist : J.n_trip;
+  for (int m = blockIdx.x * (RT / 32) + (threadIdx.x >> 5); m < n; m += nw) {
+    const int t = J.list ? J.list[m] : m;
     Comp p{0.0, 0.0}, p5{0.0, 0.0};
+    double margin = 0.0;
     double *pp = J.partial + 2LL * t * J.items_per_trip;
     for (int c = lane; c < J.items_per_trip; c += 32) {
       const double2 x = *(const double2 *)(pp + 2 * c);
       neumaier_add(p, x.x);
       neumaier_add(p5, x.y);
+      if (J.margin) margin += J.margin[(long long)t * J.items_per_trip + c];
     }
     p = warp_combine(p);
     p5 = warp_combine(p5);
+    if (J.margin) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) margin += __shfl_down_sync(0xffffffffu, margin, off);
+      if (lane == 0 && !(margin >= 0.0)) J.weak[atomicAdd(J.weak_n, 1)] = t;
+    }
     __syncwarp();                                           // every lane's reads are done
     if (lane == 0) {
       const int4 tr = J.trip[t];
@@ -99,6 +109,7 @@ __global__ void __launch_bounds__(RT) reduce_jobs(const __grid_constant__ RedBat
       J.out[0] = a.s + a.c;
       J.out[1] = absum;
       J.out[2] = a5.s + a5.c;
+      J.out[3] = J.margin ? (double)*J.weak_n : 0.0;
     }
   }
 }
@@ -108,7 +119,10 @@ __global__ void __launch_bounds__(RT) reduce_jobs(const __grid_constant__ RedBat
 cudaError_t launch_reduce(const RedBatch &b, cudaStream_t st) {
   if (b.njobs <= 0) return cudaSuccess;
   int most = 0;
-  for (int j = 0; j < b.njobs; ++j) most = b.job[j].n_trip > most ? b.job[j].n_trip : most;
+  for (int j = 0; j < b.njobs; ++j) {
+    const int n = b.job[j].list ? b.job[j].nlist : b.job[j].n_trip;
+    most = n > most ? n : most;
+  }
   if (most > 0) {
     const int blocks = (most + RT / 32 - 1) / (RT / 32);
     reduce_triplets<<<dim3(blocks < 1024 ? blocks : 1024, b.njobs), RT, 0, st>>>(b);

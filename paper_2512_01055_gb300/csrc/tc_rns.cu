@@ -50,6 +50,13 @@
 // Energy kernel.  Per tile orbit (edge 8) it loads the six W blocks as
 // integers and evaluates the canonical points in FP64: the brackets of Eq. 1
 // are differences of W, formed exactly in integers before conversion.
+//
+// Weak triplets.  The grid is common to all triplets, so W of one whose
+// amplitudes or integrals are far below the others' keeps fewer bits, where FP64
+// accumulation keeps them relative to each product.  The energy kernel therefore
+// sums, beside E[4]_ST, what E[4]_ST would be if W had WEAK_RMS units of its
+// 64-bit fraction everywhere, and the DMMA kernel forms the triplets below that
+// again.
 #include <algorithm>
 #include <type_traits>
 
@@ -89,6 +96,14 @@ constexpr int SMEM_DYN_MAX = 232448 - 2048;
 constexpr int NT = 8;                        // tile edge of the energy orbits
 constexpr int NT2 = NT * NT, NT3 = NT2 * NT;
 constexpr int EN_THREADS = 128, EN_CTAS = 5;   // per CTA, CTAs per SM
+// W is off by about 2^2.4 units where the operands have full-size norms, and on
+// data of uniform size its rms is above 2^53 units (2^57 and 2^56 per operand norm
+// less a bit each for powers of two, over sqrt(K); no triplet below 2^53 in 50
+// shapes from o=2 v=9 to o=2 v=504 and o=6 v=290): 2^-51 to 2^-53 of it, as the
+// DMMA kernel's.  WEAK_RMS is the least rms the residues are trusted with, an
+// error of 2^-49.6.  The bracket sum n4 of independent W of variance 1 has mean 72.
+constexpr double WEAK_RMS = 0x1p52;
+constexpr double WEAK_N4 = 72.0 * WEAK_RMS * WEAK_RMS;
 
 constexpr int ERR_TIMEOUT_FULL = 11, ERR_TIMEOUT_EMPTY = 12, ERR_TIMEOUT_ACCFULL = 13,
               ERR_TIMEOUT_ACCEMPTY = 14, ERR_TIMEOUT_TEARDOWN = 15;
@@ -1063,6 +1078,14 @@ __device__ __forceinline__ double recip(double x) {
   return ex - 523u <= 1000u ? rcp_fast(x) : 1.0 / x;
 }
 
+// |x| as a float (its leading 20 bits; beyond the float range 0 or infinity),
+// without the FP64 pipe.
+__device__ __forceinline__ float abs_float(double x) {
+  const int h = (__double2hiint(x) & 0x7FFFFFFF) - (896 << 20);
+  return __int_as_float(min(max(h, 0), 255 << 20) << 3);
+}
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }   // |e| <= 126
+
 // A 128-bit integer as a double (rounded once).
 __device__ __forceinline__ double u128_double(unsigned __int128 x) {
   unsigned long long h = (unsigned long long)(x >> 64);
@@ -1083,6 +1106,7 @@ __device__ __forceinline__ double u128_double(unsigned __int128 x) {
 // values take the same formulas in FP64), converted once each.  Then
 // sum_s w_s br_s = (sum_s br_s^2) / 3 - 6 d^2, formed in 128-bit integers (the
 // integer pipes have room beside the FP64 pipe); 37 FP64 operations a point in all.
+// The weak triplets' bound, WEAK_N4 times the sum of |1/D|, is summed in FP32.
 // Five small CTAs on an SM keep the pipe fed while one of them loads.
 // Orbits with equal tiles list their canonical points (36 x 8 of 512 points for
 // two equal tiles, 120 for three), so no warp runs for points outside them.
@@ -1091,6 +1115,7 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
   __shared__ long long Wb[6 * WBLK];
   __shared__ double Gs[18 * NT2], Ts[9 * NT], Eab[NT2];   // Eab: e_i + e_j + e_k - e_a - e_b
   __shared__ double s_red[EN_THREADS / 32][2];
+  __shared__ float s_abs[EN_THREADS / 32];
   __shared__ unsigned short tab2[36], tab3[120];   // points a >= b (a 8 + b) and a >= b >= c (a 64 + b 8 + c)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int e = tid; e < NT3; e += EN_THREADS) {
@@ -1116,6 +1141,7 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
     const long long *Y = J.y + (size_t)tl * v * v * vc;
     // the sums in units of the grid 2^-S of the orbits so far (S: sprev)
     double acc4 = 0.0, acc5 = 0.0;
+    float accr = 0.f;                              // sum of |1/D|
     int sprev = 0;
     const int ob0 = chunk * d.orb_per_item, ob1 = min(d.n_orb, ob0 + d.orb_per_item);
     for (int ob = ob0; ob < ob1; ++ob) {
@@ -1171,6 +1197,7 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
         const double f = __longlong_as_double((long long)(1023 + S0 - sprev) << 52);
         acc5 *= f;
         acc4 = acc4 * f * f;
+        accr *= pow2f(S0 - sprev) * pow2f(S0 - sprev);
         sprev = S0;
       }
       const bool eqP = t3[0] == t3[1], eqR = t3[1] == t3[2];
@@ -1243,6 +1270,9 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
           const double f = __longlong_as_double((long long)(1023 + dS) << 52);
           n4 = n4 * f * f;
           n5 *= f;
+          accr = fmaf(abs_float(r), pow2f(dS) * pow2f(dS), accr);
+        } else {
+          accr += abs_float(r);
         }
         acc5 = fma(n5, r, acc5);
         acc4 = fma(n4, r, acc4);
@@ -1253,18 +1283,21 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
     for (int off = 16; off > 0; off >>= 1) {
       acc4 += __shfl_down_sync(0xffffffffu, acc4, off);
       acc5 += __shfl_down_sync(0xffffffffu, acc5, off);
+      accr += __shfl_down_sync(0xffffffffu, accr, off);
     }
-    if (lane == 0) { s_red[warp][0] = acc4; s_red[warp][1] = acc5; }
+    if (lane == 0) { s_red[warp][0] = acc4; s_red[warp][1] = acc5; s_abs[warp] = accr; }
     __syncthreads();
     if (tid == 0) {
-      double e4 = 0.0, e5 = 0.0;
-      for (int k = 0; k < EN_THREADS / 32; ++k) { e4 += s_red[k][0]; e5 += s_red[k][1]; }
+      double e4 = 0.0, e5 = 0.0, er = 0.0;
+      for (int k = 0; k < EN_THREADS / 32; ++k) { e4 += s_red[k][0]; e5 += s_red[k][1]; er += s_abs[k]; }
       const double f = __longlong_as_double((long long)(1023 - sprev) << 52);
+      er = (fabs(e4) - WEAK_N4 * er) * f * (C_P * C_P / 3.0) * f;
       e4 = e4 * f * (C_P * C_P / 3.0) * f;
       e5 = e5 * f * C_P;
       const long long idx = (long long)(J.t0 + tl) * d.items_per_trip + chunk;
       J.partial[2 * idx] = e4 + e5;
       J.partial[2 * idx + 1] = e5;
+      J.margin[idx] = er;
     }
   }
 }
@@ -1377,7 +1410,8 @@ RnsGeom rns_geom(int o, int v) {
   return g;
 }
 
-RnsLayout rns_layout(int o, int v, int n_trip) {
+RnsLayout rns_layout(const Dims &d) {
+  const int o = d.o, v = d.v;
   RnsLayout L{};
   const RnsGeom g = rns_geom(o, v);
   L.g = g;
@@ -1397,9 +1431,11 @@ RnsLayout rns_layout(int o, int v, int n_trip) {
   L.rt = take(O * V * V * 8);
   L.rb = take(O * O * V * 8);
   L.rh = take(O * V * O * 8);
-  L.mx = take(4 * (V + O) * 8);
+  L.mx = take((4 * (V + O) + 1) * 8);
   L.ex = take((3 * (V + O) + 8) * 4);
-  L.unit = take((size_t)3 * std::max(1, n_trip) * 4);
+  L.unit = take((size_t)3 * std::max(1, d.n_trip) * 4);
+  L.margin = take((size_t)std::max<long long>(1, d.n_items) * 8);
+  L.weak = take((size_t)std::max(1, d.n_trip) * 4);
   L.need = take(O * O);
   L.total = off;
   return L;
@@ -1434,7 +1470,8 @@ cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, cons
   const Scales s = scales_at(L, ws, flag);
   cudaError_t e = cudaMemcpyAsync(b + L.unit, t.unit.data(), t.unit.size() * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !all) e = cudaMemcpyAsync(b + L.need, t.need.data(), t.need.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b + L.mx, 0, 4 * ((size_t)g.v + g.o) * 8, st);
+  // the maxima and the number of weak triplets behind them
+  if (e == cudaSuccess) e = cudaMemsetAsync(b + L.mx, 0, (4 * ((size_t)g.v + g.o) + 1) * 8, st);
   if (e != cudaSuccess) return e;
   const unsigned char *need = all ? nullptr : (const unsigned char *)(b + L.need);
   rns_norms<<<PREP_BLOCKS, PREP_THREADS, 4 * ((size_t)g.v + g.o) * 8, st>>>(in, g.o, g.v, s);
@@ -1488,8 +1525,16 @@ void rns_block(const RnsLayout &L, void *ws, const Dims &d, const Inputs &in, co
   E.uo = s.uo;
   E.sh = s.sh;
   E.partial = w.partial;
+  E.margin = (double *)(b + L.margin);
   E.t0 = t0;
   E.nt = nt;
+}
+
+void rns_weak(const RnsLayout &L, void *ws, RedJob *j) {
+  char *b = (char *)ws;
+  j->margin = (const double *)(b + L.margin);
+  j->weak_n = (int *)(b + L.mx + 4 * ((size_t)L.g.v + L.g.o) * 8);
+  j->weak = (int *)(b + L.weak);
 }
 
 cudaError_t rns_block_params(RnBatch *gb, RnEnBatch &eb, int num_sms, void **gargs, void **eargs,

@@ -64,6 +64,7 @@ struct Req {
   bool waited = false;                    // the compute stream waits on `ready` once
   long long units = 0;                    // work units: FP64 items, or split-path triplets
   long long next_item = 0;                // next unit to run
+  int nweak = 0;                          // > 0: group 0 forms these triplets of a G_RNS job again
   double cost_per_item = 1.0;             // cost of one unit
   St state = St::Queued;
   tc_status status = TC_OK;
@@ -129,8 +130,15 @@ int gemm_launches(int g) { return g == 0 ? 1 : g == G_RNS ? RNS_GEMM_LAUNCHES : 
 // of the DMMA kernel, else a whole triplet.
 void set_units(Req &q) {
   const bool items = q.group == 0;
-  q.units = items ? q.d.n_items : q.d.n_trip;
+  q.units = items ? (q.nweak > 0 ? (long long)q.nweak * q.d.items_per_trip : q.d.n_items) : q.d.n_trip;
   q.cost_per_item = (double)(items ? q.d.orb_per_item : q.d.n_orb) * (q.v + 16.0 * ((q.o + 15) / 16));
+}
+
+// The reduction's fields for the weak triplets of a job of the tensor-core group.
+RedJob weak_job(Req &q) {
+  RedJob j{};
+  rns_weak(q.RL, q.mem + q.off_split, &j);
+  return j;
 }
 
 }  // namespace
@@ -346,7 +354,7 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
     for (int j = 0; j < nj; ++j) {
       Req &q = *jobs[j];
       const Inputs in{q.din[0], q.din[1], q.din[2], q.din[3], q.din[4], q.din[5]};
-      fb.job[j] = FpJob{q.d, in, q.w, total, q.next_item};
+      fb.job[j] = FpJob{q.d, in, q.w, total, q.next_item, q.nweak > 0 ? weak_job(q).weak : nullptr};
       total += take[j];
       cost += take[j] * q.cost_per_item;
     }
@@ -433,7 +441,8 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
   return true;
 }
 
-// Multi-job reduction of the jobs whose last items ran, then completion.
+// Multi-job reduction of the jobs whose last items ran, then completion; FP64
+// jobs with triplets too weak for the common grid go on to the DMMA group.
 void Server::finish(std::vector<std::shared_ptr<Req>> &done) {
   for (size_t b0 = 0; b0 < done.size(); b0 += MAX_BATCH) {
     const int n = (int)std::min<size_t>(MAX_BATCH, done.size() - b0);
@@ -442,16 +451,31 @@ void Server::finish(std::vector<std::shared_ptr<Req>> &done) {
     for (int j = 0; j < n; ++j) {
       Req &q = *done[b0 + j];
       char *base = q.mem + q.off_ws;
-      rb.job[j] = RedJob{q.d.n_trip, q.d.items_per_trip, q.o, q.w.trip, q.w.partial,
-                         (double *)(base + q.L.e_trip), nullptr, d_out + 4 * j};
+      RedJob &J = rb.job[j];
+      J = RedJob{q.d.n_trip, q.d.items_per_trip, q.o, q.w.trip, q.w.partial,
+                 (double *)(base + q.L.e_trip), nullptr, d_out + 4 * j};
+      if (q.group == G_RNS) {
+        rns_weak(q.RL, q.mem + q.off_split, &J);
+      } else if (q.nweak > 0) {
+        J.list = weak_job(q).weak;
+        J.nlist = q.nweak;
+      }
     }
     cudaError_t e = launch_reduce(rb, compute);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_out, d_out, sizeof(double) * 4 * n, cudaMemcpyDeviceToHost, compute);
-    for (int j = 0; j < n; ++j) cudaFreeAsync(done[b0 + j]->mem, compute);
     if (e == cudaSuccess) e = cudaStreamSynchronize(compute);
     std::lock_guard<std::mutex> lk(mu);
     for (int j = 0; j < n; ++j) {
       auto &r = done[b0 + j];
+      if (e == cudaSuccess && r->group == G_RNS && h_out[4 * j + 3] > 0.0) {
+        r->nweak = (int)h_out[4 * j + 3];
+        r->group = 0;
+        r->next_item = 0;
+        set_units(*r);
+        r->state = St::Ready;
+        continue;
+      }
+      cudaFreeAsync(r->mem, compute);
       r->mem = nullptr;
       reserved -= r->footprint;
       active.erase(std::find(active.begin(), active.end(), r));
@@ -641,7 +665,7 @@ tc_status tc_submit(tc_ctx *ctx, const tc_job *job, uint64_t *ticket) {
   // FP64 on the tensor cores as in the blocking entry points, within a quarter
   // of the budget so that other jobs are admitted beside it
   if (!split && r->d.n_trip > 0 && tc::rns_supported(o, v)) {
-    r->RL = tc::rns_layout(o, v, r->d.n_trip);
+    r->RL = tc::rns_layout(r->d);
     if (r->RL.total <= ctx->budget / 4) r->group = tc::G_RNS;
     else r->RL = tc::RnsLayout{};
   }

@@ -54,11 +54,10 @@ def _scale(d, what, k):
     d = {n: x.clone() for n, x in d.items()}
     f, p, x = 2.0 ** -k, 2, 5
     ints = what.startswith("ints")
-    if what == "t2_fragments":                      # pairs between {0, 1} and the rest, and two virtual blocks
-        d["t2"][:2, 2:] *= f
-        d["t2"][2:, :2] *= f
-        d["t2"][:, :, :9, 9:] *= f
-        d["t2"][:, :, 9:, :9] *= f
+    if what == "pairs":                             # weakly coupled orbitals: triplets of three are weak, others are not
+        keep = torch.eye(o, dtype=torch.bool, device="cuda")[:, :, None, None]
+        d["t2"] = torch.where(keep, d["t2"], d["t2"] * f)
+        d["ovoo"] *= f
         return d
     if what in ("ovvv_occ", "ints_occ"):
         d["ovvv"][p] *= f
@@ -98,3 +97,41 @@ def test_operands_of_one_orbital_smaller_than_the_others(what, k):
     print(f"{what} 2^-{k}: max |de| / max |e| = {np.abs(e - ref).max() / scale:.2e}, dE/E = {abs(r.e_t / e_ref - 1):.2e}")
     assert np.abs(e - ref).max() <= 1e-12 * scale
     assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
+
+
+# A triplet's W is right to 2^-49 of its own size (the weakest the residues are used for), the reference's to 2^-50;
+# e_ijk may cancel between its W and V parts: three orders of magnitude over that.
+@pytest.mark.parametrize("what", WHAT + ["pairs"])
+@pytest.mark.parametrize("k", [6, 12, 20, 30])
+def test_every_triplet_keeps_its_own_digits(what, k):
+    o, v = 6, 21
+    d = _scale(_random(o, v, 612), what, k)
+    r, e = _energy(o, v, d)
+    assert r.prep_seconds > 0.0
+    e_ref, ref = _noalloc(o, v, d)
+    nz = ref != 0.0
+    worst = np.abs(e[nz] / ref[nz] - 1).max()
+    print(f"{what} 2^-{k}: worst relative error of a triplet {worst:.2e}")
+    assert worst <= 1e-11
+    assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
+
+
+def test_served_job_with_weak_triplets():
+    """A job some of whose triplets are formed again gives the same bits alone and served, beside one with none."""
+    jobs = [(6, 21, _scale(_random(6, 21, 612), "pairs", 20)), (5, 24, _random(5, 24, 613))]
+    alone = [_energy(*j)[0] for j in jobs]
+    strong = _energy(6, 21, _random(6, 21, 612))[0]
+    assert alone[0].launches > strong.launches                       # some triplets were weak
+    ctx = tc.tc_init(0, max_inflight=4)
+    try:
+        for _ in range(2):
+            tickets = [tc.tc_submit(ctx, o, v, d["eps"], d["t1"], d["t2"], d["ovvv"], d["ovoo"], d["ovov"],
+                                    prec=tc.TC_FP64, device_inputs=True) for o, v, d in jobs]
+            for t, a in zip(tickets, alone):
+                code, r = tc.tc_wait(ctx, t, 60000)
+                assert code == tc.TC_OK
+                assert r.e_t == a.e_t and r.e_t5 == a.e_t5
+        st = tc.tc_serve_stats_get(ctx)
+        assert st.completed == 4 and st.failed == 0 and st.reserved_bytes == 0 and st.inflight == 0
+    finally:
+        tc.tc_finalize(ctx)
