@@ -216,6 +216,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
         const int t0 = blk * nb, nt = std::min(nb, d.n_trip - t0);
         gb[0].njobs = gb[1].njobs = eb.njobs = 1;
         gb[0].err = gb[1].err = w.err;
+        gb[0].skip = gb[1].skip = eb.skip = w.err + 1;
         tc::rns_block(RL, ctx->ws_rns.p, d, in, w, rt, t0, nt, &gb[0].job[0], &gb[1].job[0], &eb.job[0]);
         TC_CUDA(ctx, tc::launch_rns_block(gb, eb, ctx->num_sms, st, ctx->wev[2 * blk], ctx->wev[2 * blk + 1]));
       }

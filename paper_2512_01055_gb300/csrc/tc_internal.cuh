@@ -220,6 +220,7 @@ struct RnBatch {
   size_t slot;           // set by the launcher: stage stride in shared memory
   long long total_items;
   int *err;
+  const int *skip;       // optional device flag: not 0, the launch does nothing (inputs beyond the integer grid)
   RnJob job[MAX_BATCH];
 };
 struct RnEnJob {         // one job's block of triplets in an energy launch
@@ -237,6 +238,7 @@ struct RnEnJob {         // one job's block of triplets in an energy launch
 struct RnEnBatch {
   int njobs;
   long long total_items;
+  const int *skip;       // as RnBatch::skip
   RnEnJob job[MAX_BATCH];
 };
 constexpr int RNS_GEMM_LAUNCHES = 2;       // storing, then adding

@@ -780,6 +780,7 @@ __device__ __forceinline__ void drain_product(int l, int my, uint32_t tacc, uint
 template <int UN>
 __global__ void __launch_bounds__(THREADS, 1)
 rns_gemm_kernel(const __grid_constant__ RnBatch B) {
+  if (B.skip && *B.skip) return;                   // the results would not be used
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *sm = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
 
@@ -1112,6 +1113,7 @@ __device__ __forceinline__ double u128_double(unsigned __int128 x) {
 // two equal tiles, 120 for three), so no warp runs for points outside them.
 __global__ void __launch_bounds__(EN_THREADS, EN_CTAS)
 rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
+  if (B.skip && *B.skip) return;
   __shared__ long long Wb[6 * WBLK];
   __shared__ double Gs[18 * NT2], Ts[9 * NT], Eab[NT2];   // Eab: e_i + e_j + e_k - e_a - e_b
   __shared__ double s_red[EN_THREADS / 32][2];

@@ -135,3 +135,16 @@ def test_served_job_with_weak_triplets():
         assert st.completed == 4 and st.failed == 0 and st.reserved_bytes == 0 and st.inflight == 0
     finally:
         tc.tc_finalize(ctx)
+
+
+def test_inputs_beyond_the_grid_do_not_run_the_residue_products():
+    """The call notices them after its preparation: what it does besides the DMMA kernel is a small part of a call."""
+    o, v = 8, 104
+    d = _random(o, v, 95)
+    good = min((_energy(o, v, d)[0] for _ in range(3)), key=lambda r: r.seconds)
+    d["ovvv"][2, 3, 4, 5] = float("inf")
+    bad = min((_energy(o, v, d)[0] for _ in range(3)), key=lambda r: r.seconds - r.kernel_seconds)
+    assert bad.prep_seconds == 0.0 and bad.kernel_seconds > 5 * good.kernel_seconds
+    print(f"good {good.seconds:.4f} s, of it residue kernels {good.kernel_seconds:.4f} s; "
+          f"beside the DMMA kernel {bad.seconds - bad.kernel_seconds:.4f} s")
+    assert bad.seconds - bad.kernel_seconds < 0.5 * good.kernel_seconds
