@@ -428,7 +428,8 @@ cudaError_t df_gemm(const DfGemm &G0, int num_sms, cudaStream_t st) {
   G.stages = (int)std::min<long long>(DF_MAX_STAGES, (long long)(DF_SMEM_MAX - 1024) / (long long)G.slot);
   if (G.stages < DF_NPROD) return cudaErrorInvalidValue;
   const size_t smem = 1024 + (size_t)G.stages * G.slot;
-  cudaError_t e = cudaFuncSetAttribute(df_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // always the same limit: it is the process's, and another thread may be between this and its launch
+  cudaError_t e = cudaFuncSetAttribute(df_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DF_SMEM_MAX);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)G.mt * G.nt;
   const int grid = (int)std::max<long long>(1, std::min<long long>(num_sms, tiles));

@@ -1379,7 +1379,9 @@ cudaError_t prepare(RnBatch *gb, RnEnBatch &eb, int num_sms, int *ggrid, int *eg
   eb.total_items = total;
   *egrid = (int)std::max<long long>(1, std::min<long long>((long long)EN_CTAS * num_sms, total));
   *fn = rn_kernel(ncmax);
-  return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  // The limit is the process's, not the launch's: always the same value, as another
+  // thread may be between this and its launch.
+  return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN_MAX);
 }
 
 }  // namespace

@@ -1207,7 +1207,8 @@ cudaError_t prepare(WtBatch &wb, EnBatch &eb, int S, int num_sms, int *wgrid, in
   *wgrid = (int)std::max<long long>(1, std::min<long long>(num_sms, total));
   *egrid = (int)std::max<long long>(1, std::min<long long>(num_sms, etotal));
   *wfn = wt_kernel(S, ncmax);
-  cudaError_t e = cudaFuncSetAttribute(*wfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
+  // always the same limit: it is the process's, and another thread may be between this and its launch
+  cudaError_t e = cudaFuncSetAttribute(*wfn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_DYN_MAX);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_energy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, EN_SMEM);
   return e;
 }
