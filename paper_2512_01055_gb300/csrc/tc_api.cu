@@ -98,10 +98,16 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   // 0.8 s (4.3 ps a byte) to the 50 s of o=40 v=400, and the DMMA kernel does
   // 0.9 flop per ps, so 12 v^4 flop a triplet against 10 flop a byte leaves a
   // factor of 2.5 (the whole energy: 71 against 1.0 TFLOP/s).
+  // Buffers of earlier calls that this one does not use give way to it.
   const tc::RnsLayout RL = split ? tc::RnsLayout{} : tc::rns_layout(d);
+  size_t unused = 0;
+  for (const tc::DevBuf *b : ctx->unused_by_fp64(in.ovvv)) unused += b->cap;
+  auto release_unused = [&] {
+    for (tc::DevBuf *b : ctx->unused_by_fp64(in.ovvv)) b->release();
+  };
   bool rns = !split && !dmma && d.n_trip > 0 && tc::rns_supported(o, v) &&
              (RL.total <= ctx->budget / 4 || 12.0 * d.n_trip * v * v * v * v >= 10.0 * RL.total) &&
-             need + RL.total + ctx->in_ovvv.cap + ctx->in_t2.cap + ctx->in_ovov.cap + ctx->in_ovoo.cap <= ctx->budget;
+             ctx->held() - ctx->ws_rns.cap - unused + RL.total <= ctx->budget;
   struct GiveBack {
     tc_ctx *ctx;
     ~GiveBack() {
@@ -112,7 +118,13 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
     }
   } give_back{ctx};
   if (rns) {
-    const cudaError_t e = ctx->ws_rns.ensure(RL.total);
+    if (ctx->held() - ctx->ws_rns.cap + RL.total > ctx->budget) release_unused();
+    cudaError_t e = ctx->ws_rns.ensure(RL.total);
+    if (e == cudaErrorMemoryAllocation && unused > 0) {
+      cudaGetLastError();
+      release_unused();
+      e = ctx->ws_rns.ensure(RL.total);
+    }
     if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
       rns = false;

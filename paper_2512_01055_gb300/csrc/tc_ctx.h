@@ -56,8 +56,24 @@ struct tc_ctx {
   cudaStream_t copy_stream = nullptr;       // tc_energy: host-to-device copies of the inputs, by occupied-index chunk
   std::vector<cudaEvent_t> cev;             // tc_energy: one per chunk, recorded on copy_stream after its copies
   std::vector<cudaEvent_t> pev;             // staged split path: a pair around each chunk's slicing
-  // Grow a buffer; when the device is out of memory, the residue images give way.
+  // Device bytes of all buffers.
+  size_t held() const {
+    size_t s = 0;
+    for (const tc::DevBuf *b : {&ws, &ws_split, &ws_rns, &in_eps, &in_t1, &in_t2, &in_ovvv, &in_ovoo, &in_ovov, &df_b, &df_in})
+      s += b->cap;
+    return s;
+  }
+  // The buffers an FP64 call on these integrals does not use: the split path's,
+  // and the inputs and factors unless the integrals are the context's own.
+  std::vector<tc::DevBuf *> unused_by_fp64(const double *ovvv) {
+    std::vector<tc::DevBuf *> u{&ws_split};
+    if (ovvv != in_ovvv.p) u.insert(u.end(), {&in_eps, &in_t1, &in_t2, &in_ovvv, &in_ovoo, &in_ovov, &df_b, &df_in});
+    return u;
+  }
+  // Grow a buffer; the residue images of earlier calls give way when the budget
+  // or the device has no room beside them.
   cudaError_t grow(tc::DevBuf &b, size_t bytes) {
+    if (&b != &ws_rns && bytes > b.cap && held() - b.cap + bytes > budget) ws_rns.release();
     cudaError_t e = b.ensure(bytes);
     if (e == cudaErrorMemoryAllocation && &b != &ws_rns && ws_rns.p) {
       cudaGetLastError();

@@ -46,3 +46,58 @@ def test_launches_of_one_kernel_with_different_shared_memory(prec, slices):
     for th in ths:
         th.join()
     assert not bad, (len(bad), bad[:2])
+
+
+def _used(free):
+    import torch
+    torch.cuda.synchronize()
+    return free - torch.cuda.mem_get_info()[0]
+
+
+SLACK = 48 << 20        # small buffers, 2 MB allocation granularity, kernels loaded on first use
+
+
+def _warm():
+    """Every kernel and the caching allocator's blocks in place, so that only contexts' buffers change the free memory."""
+    d = _random(3, 24, 9)
+    ctx = tc.tc_init(0)
+    for prec in (tc.TC_FP64, tc.TC_SPLIT_BF16):
+        tc.tc_energy_dev(ctx, 3, 24, *_args(d), prec=prec, slices=4)
+        code, _ = tc.tc_wait(ctx, tc.tc_submit(ctx, 3, 24, *_args(d), prec=prec, slices=4, device_inputs=True), 60000)
+        assert code == tc.TC_OK
+    tc.tc_finalize(ctx)
+
+
+def test_residue_images_and_the_buffers_of_earlier_calls():
+    """Split images of most of the budget, then an FP64 call, then a split call again: the context never holds more
+    than the budget, and each call runs on its own path."""
+    import torch
+    small, large = _random(4, 64, 64), _random(10, 128, 65)
+    need = tc.tc_workspace_bytes(10, 128, tc.TC_SPLIT_BF16, 4)
+    budget = need + (32 << 20)                        # the images of o=4 v=64 take about 115 MB
+    _warm()
+    free = torch.cuda.mem_get_info()[0]
+    ctx = tc.tc_init(0, hbm_budget_bytes=budget)
+    try:
+        for _ in range(2):
+            tc.tc_energy_dev(ctx, 10, 128, *_args(large), prec=tc.TC_SPLIT_BF16, slices=4)
+            print(f"budget {budget >> 20} MB, used after the split call {_used(free) >> 20} MB")
+            assert _used(free) <= budget + SLACK
+            r = tc.tc_energy_dev(ctx, 4, 64, *_args(small), prec=tc.TC_FP64)
+            assert r.prep_seconds > 0.0 and 64 << 20 < _used(free) <= budget + SLACK      # residues, kept
+    finally:
+        tc.tc_finalize(ctx)
+
+
+def test_residue_images_beside_the_context_s_own_inputs():
+    """A host call's inputs are in use: with no room for the images beside them the DMMA kernel runs."""
+    d = _random(4, 64, 64)
+    host = [x.cpu().numpy() for x in _args(d)]
+    inputs = sum(x.nbytes for x in host)
+    for extra, dmma in ((64 << 20, True), (256 << 20, False)):
+        ctx = tc.tc_init(0, hbm_budget_bytes=inputs + extra)
+        try:
+            r = tc.tc_energy(ctx, 4, 64, *host, prec=tc.TC_FP64)
+            assert (r.prep_seconds == 0.0) == dmma
+        finally:
+            tc.tc_finalize(ctx)
