@@ -100,31 +100,36 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   // factor of 2.5 (the whole energy: 71 against 1.0 TFLOP/s).
   // Buffers of earlier calls that this one does not use give way to it.
   const tc::RnsLayout RL = split ? tc::RnsLayout{} : tc::rns_layout(d);
-  size_t unused = 0;
+  size_t unused = 0, served = 0;
+  if (!split) {
+    std::lock_guard<std::mutex> lk(ctx->serve_mu);
+    if (ctx->server) served = tc::server_reserved(ctx->server);
+  }
   for (const tc::DevBuf *b : ctx->unused_by_fp64(in.ovvv)) unused += b->cap;
   auto release_unused = [&] {
     for (tc::DevBuf *b : ctx->unused_by_fp64(in.ovvv)) b->release();
   };
   bool rns = !split && !dmma && d.n_trip > 0 && tc::rns_supported(o, v) &&
              (RL.total <= ctx->budget / 4 || 12.0 * d.n_trip * v * v * v * v >= 10.0 * RL.total) &&
-             ctx->held() - ctx->ws_rns.cap - unused + RL.total <= ctx->budget;
+             ctx->held() - ctx->ws_rns.cap - unused + served + RL.total <= ctx->budget;
   struct GiveBack {
     tc_ctx *ctx;
     ~GiveBack() {
       if (ctx->ws_rns.cap > ctx->budget / 4) {
         cudaDeviceSynchronize();                         // an early return may leave kernels in flight
-        ctx->ws_rns.release();
+        ctx->release_rns();
       }
     }
   } give_back{ctx};
   if (rns) {
-    if (ctx->held() - ctx->ws_rns.cap + RL.total > ctx->budget) release_unused();
+    if (ctx->held() - ctx->ws_rns.cap + served + RL.total > ctx->budget) release_unused();
     cudaError_t e = ctx->ws_rns.ensure(RL.total);
     if (e == cudaErrorMemoryAllocation && unused > 0) {
       cudaGetLastError();
       release_unused();
       e = ctx->ws_rns.ensure(RL.total);
     }
+    ctx->rns_held = ctx->ws_rns.p != nullptr;
     if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
       rns = false;

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -27,6 +28,7 @@ struct DevBuf {
 
 struct Server;                              // serving engine (tc_serve.cu)
 void server_destroy(Server *s);
+size_t server_reserved(Server *s);          // device bytes held by admitted jobs
 
 }  // namespace tc
 
@@ -70,18 +72,23 @@ struct tc_ctx {
     if (ovvv != in_ovvv.p) u.insert(u.end(), {&in_eps, &in_t1, &in_t2, &in_ovvv, &in_ovoo, &in_ovov, &df_b, &df_in});
     return u;
   }
-  // Grow a buffer; the residue images of earlier calls give way when the budget
+  // Grow a buffer other than ws_rns; the residue images of earlier calls give way when the budget
   // or the device has no room beside them.
   cudaError_t grow(tc::DevBuf &b, size_t bytes) {
-    if (&b != &ws_rns && bytes > b.cap && held() - b.cap + bytes > budget) ws_rns.release();
+    if (bytes > b.cap && held() - b.cap + bytes > budget) release_rns();
     cudaError_t e = b.ensure(bytes);
-    if (e == cudaErrorMemoryAllocation && &b != &ws_rns && ws_rns.p) {
+    if (e == cudaErrorMemoryAllocation && ws_rns.p) {
       cudaGetLastError();
-      ws_rns.release();
+      release_rns();
       e = b.ensure(bytes);
     }
     return e;
   }
+  void release_rns() {
+    ws_rns.release();
+    rns_held = false;
+  }
+  std::atomic<bool> rns_held{false};        // ws_rns holds memory (read by the server without mu)
   std::mutex serve_mu;                      // guards creation of the serving engine
   tc::Server *server = nullptr;
 };

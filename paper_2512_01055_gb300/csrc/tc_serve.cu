@@ -180,10 +180,30 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
   const bool split = q.prec == TC_SPLIT_BF16;
   cudaError_t e = cudaSuccess;
   if (q.inject_alloc_fault) e = cudaErrorMemoryAllocation;
-  if (e == cudaSuccess) e = cudaMallocAsync((void **)&q.mem, q.footprint, q.st);
+  // Residue images that a blocking FP64 call left in the context give way: when
+  // the budget has no room beside them, and below when the device has none.
+  {
+    std::unique_lock<std::mutex> calls(ctx->mu, std::try_to_lock);
+    if (calls && ctx->ws_rns.p) {
+      std::lock_guard<std::mutex> lk(mu);
+      if (reserved + ctx->ws_rns.cap > ctx->budget) ctx->release_rns();
+    }
+  }
+  auto alloc = [&] {
+    const cudaError_t a = cudaMallocAsync((void **)&q.mem, q.footprint, q.st);
+    if (a == cudaErrorMemoryAllocation) cudaGetLastError();
+    return a;
+  };
+  if (e == cudaSuccess) e = alloc();
+  if (e == cudaErrorMemoryAllocation && !q.inject_alloc_fault) {
+    std::unique_lock<std::mutex> calls(ctx->mu, std::try_to_lock);
+    if (calls && ctx->ws_rns.p) {
+      ctx->release_rns();
+      e = alloc();
+    }
+  }
   if (e == cudaErrorMemoryAllocation && !q.inject_alloc_fault && q.group == G_RNS) {
     // no room for the residue images: the job runs on the DMMA kernel
-    cudaGetLastError();
     {
       std::lock_guard<std::mutex> lk(mu);
       reserved -= q.RL.total;
@@ -191,7 +211,13 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
       q.group = 0;
       set_units(q);
     }
-    e = cudaMallocAsync((void **)&q.mem, q.footprint, q.st);
+    e = alloc();
+  }
+  if (e == cudaErrorMemoryAllocation && !q.inject_alloc_fault && ctx->rns_held) {
+    // the images of a blocking call under way: wait for its end
+    std::lock_guard<std::mutex> calls(ctx->mu);
+    ctx->release_rns();
+    e = alloc();
   }
   if (e != cudaSuccess) {
     q.mem = nullptr;
@@ -583,6 +609,11 @@ void Server::sched_loop() {
     }
     lk.lock();
   }
+}
+
+size_t server_reserved(Server *s) {
+  std::lock_guard<std::mutex> lk(s->mu);
+  return s->reserved;
 }
 
 void server_destroy(Server *s) {

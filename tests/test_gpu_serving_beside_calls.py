@@ -1,4 +1,5 @@
 """Served jobs and blocking calls side by side on one device: launch limits, memory, waiting.  Nothing is faulted."""
+import ctypes
 import threading
 import time
 
@@ -57,6 +58,14 @@ def _used(free):
 SLACK = 48 << 20        # small buffers, 2 MB allocation granularity, kernels loaded on first use
 
 
+def _trim():
+    """Give the device's memory pool, which keeps served jobs' memory for reuse, back to the device."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool = ctypes.c_void_p()
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    assert cu.cuMemPoolTrimTo(pool, ctypes.c_size_t(0)) == 0
+
+
 def _warm():
     """Every kernel and the caching allocator's blocks in place, so that only contexts' buffers change the free memory."""
     d = _random(3, 24, 9)
@@ -66,6 +75,7 @@ def _warm():
         code, _ = tc.tc_wait(ctx, tc.tc_submit(ctx, 3, 24, *_args(d), prec=prec, slices=4, device_inputs=True), 60000)
         assert code == tc.TC_OK
     tc.tc_finalize(ctx)
+    _trim()
 
 
 def test_residue_images_and_the_buffers_of_earlier_calls():
@@ -101,3 +111,48 @@ def test_residue_images_beside_the_context_s_own_inputs():
             assert (r.prep_seconds == 0.0) == dmma
         finally:
             tc.tc_finalize(ctx)
+
+
+def test_kept_residue_images_give_way_to_served_jobs_in_the_budget():
+    """Images kept after a blocking FP64 call, then a served job of nearly the whole budget."""
+    import torch
+    small, large = _random(4, 64, 64), _random(10, 128, 65)
+    budget = tc.tc_workspace_bytes(10, 128, tc.TC_SPLIT_BF16, 4) + (32 << 20)
+    _warm()
+    free = torch.cuda.mem_get_info()[0]
+    ctx = tc.tc_init(0, hbm_budget_bytes=budget)
+    try:
+        r = tc.tc_energy_dev(ctx, 4, 64, *_args(small), prec=tc.TC_FP64)
+        assert r.prep_seconds > 0.0 and _used(free) > 64 << 20
+        t = tc.tc_submit(ctx, 10, 128, *_args(large), prec=tc.TC_SPLIT_BF16, slices=4, device_inputs=True)
+        code, _ = tc.tc_wait(ctx, t, 60000)
+        assert code == tc.TC_OK
+        print(f"budget {budget >> 20} MB, used {_used(free) >> 20} MB")       # the pool keeps the job's memory
+        assert _used(free) <= budget + SLACK
+    finally:
+        tc.tc_finalize(ctx)
+
+
+@pytest.mark.parametrize("prec,slices", [(tc.TC_SPLIT_BF16, 4), (tc.TC_FP64, 0)])
+def test_kept_residue_images_give_way_to_served_jobs_on_a_full_device(prec, slices):
+    """The device has less room than the budget: the job that fits once the images are given back runs.  (FP64 with
+    its own images of the same size: it takes the room rather than the DMMA kernel.)"""
+    import torch
+    large = _random(10, 128, 65)
+    ctx = tc.tc_init(0, hbm_budget_bytes=8 << 30)
+    fill = None
+    try:
+        ref = tc.tc_energy_dev(ctx, 10, 128, *_args(large), prec=tc.TC_FP64)      # about 1.3 GB of images, kept
+        assert ref.prep_seconds > 0.0
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        _trim()
+        fill = torch.empty(torch.cuda.mem_get_info()[0] - (768 << 20), dtype=torch.uint8, device="cuda")
+        t = tc.tc_submit(ctx, 10, 128, *_args(large), prec=prec, slices=slices, device_inputs=True)
+        code, r = tc.tc_wait(ctx, t, 60000)
+        assert code == tc.TC_OK
+        if prec == tc.TC_FP64:
+            assert r.e_t == ref.e_t
+    finally:
+        del fill
+        tc.tc_finalize(ctx)
