@@ -242,8 +242,9 @@ tc_status tc_combine_parts(const double *parts, int n, double *e_t);
  * streams while others compute.  Computation proceeds in iterations of about
  * iteration_ms: each iteration is one persistent multi-job launch (replayed
  * from a CUDA graph) over a slice of the items of every ready job of one
- * precision group (a small batch first waits for a small job of its group that
- * is being handed in or prepared), the slices shared fairly, so a job submitted while others
+ * precision group (a small batch first waits, a quarter of iteration_ms at most,
+ * for a small job of its group that is being handed in or prepared), the slices
+ * shared fairly, so a job submitted while others
  * run starts within an iteration and small jobs are not stuck behind large
  * ones.  A job's result does not depend on the other jobs it ran with.
  * ------------------------------------------------------------------------ */

@@ -565,7 +565,8 @@ void Server::sched_loop() {
       }
     }
     // pick the next group (round robin) that has ready work and whose batch is
-    // not about to grow; it waits for that a few iterations' time at most
+    // not about to grow; it waits for that a quarter of an iteration at most
+    // (with clients that keep submitting a batch is always about to grow)
     std::vector<std::shared_ptr<Req>> jobs;
     int g = -1;
     bool waits = false;
@@ -578,7 +579,7 @@ void Server::sched_loop() {
       if (batch_may_grow(gg, jobs)) {
         const auto now = Clock::now();
         if (!lingering[gg]) { lingering[gg] = true; t_linger[gg] = now; }
-        if (now - t_linger[gg] < std::chrono::milliseconds(4 * ctx->iteration_ms)) {
+        if (now - t_linger[gg] < std::chrono::microseconds(250LL * ctx->iteration_ms)) {
           waits = true;
           jobs.clear();
           continue;

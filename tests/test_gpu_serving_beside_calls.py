@@ -156,3 +156,41 @@ def test_kept_residue_images_give_way_to_served_jobs_on_a_full_device(prec, slic
     finally:
         del fill
         tc.tc_finalize(ctx)
+
+
+def test_first_job_starts_while_clients_keep_handing_in():
+    """Twelve clients hand in small host jobs without a pause for 1.5 s (most are refused: the queue is short), so a
+    batch is always about to grow: the first job starts after a quarter of an iteration, 0.25 s, not when the clients
+    are done."""
+    d = _random(3, 120, 66)
+    host = [x.cpu().numpy() for x in _args(d)]
+    ctx = tc.tc_init(0, iteration_ms=1000, max_inflight=4, max_queue=8)
+    tickets, lock = [], threading.Lock()
+
+    def client(end):
+        while time.monotonic() < end:
+            try:
+                t = tc.tc_submit(ctx, 3, 120, *host, prec=tc.TC_SPLIT_BF16, slices=3)
+            except tc.TcError as e:
+                assert e.status == tc.TC_EBUSY
+                continue
+            with lock:
+                tickets.append(t)
+
+    try:
+        code, _ = tc.tc_wait(ctx, tc.tc_submit(ctx, 3, 120, *host, prec=tc.TC_SPLIT_BF16, slices=3), 60000)
+        assert code == tc.TC_OK                                         # threads, kernels and pool are in place
+        ths = [threading.Thread(target=client, args=(time.monotonic() + 1.5,)) for _ in range(12)]
+        for th in ths:
+            th.start()
+        for th in ths:
+            th.join()
+        done = {}
+        for t in tickets:
+            code, done[t] = tc.tc_wait(ctx, t, 120000)
+            assert code == tc.TC_OK
+        first = done[min(done)].queue_seconds
+        print(f"{len(tickets)} jobs taken, the first started after {first:.3f} s")
+        assert first < 0.75
+    finally:
+        tc.tc_finalize(ctx)
