@@ -79,8 +79,8 @@ struct FpBatch {
 };
 int fp64_tile();
 size_t fp64_smem_bytes();
-cudaError_t fp64_blocks_per_sm(int *n);
-cudaError_t launch_fp64(const FpBatch &b, int grid, cudaStream_t st);
+[[nodiscard]] cudaError_t fp64_blocks_per_sm(int *n);
+[[nodiscard]] cudaError_t launch_fp64(const FpBatch &b, int grid, cudaStream_t st);
 // Kernel-node parameters of one FP64 launch (for CUDA graphs); args[0] must
 // point to b while the parameters are used.
 void fp64_node_params(const FpBatch &b, int grid, void **args, cudaKernelNodeParams *p);
@@ -154,27 +154,28 @@ SplitLayout split_layout(int o, int v, int S);
 // and launch_split_prep_range those read from t2, ovvv, ovoo and ovov rows
 // whose first occupied index lies in [p0, p1) (what a triplet (i, j, k) with
 // i >= j >= k reads lies in the rows p <= i).
-cudaError_t launch_split_prep(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st);
-cudaError_t launch_split_prep_common(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st);
-cudaError_t launch_split_prep_range(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st, int p0, int p1);
+[[nodiscard]] cudaError_t launch_split_prep(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_split_prep_common(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_split_prep_range(const SplitLayout &L, const Inputs &in, void *ws, cudaStream_t st,
+                                                  int p0, int p1);
 int split_prep_launches();
 int split_prep_common_launches();
 int split_prep_range_launches();
 WtJob wt_job(const SplitLayout &L, const void *ws, const int4 *trip, int t0, int nt);
 // Energy job of triplets [t0, t0 + nt); encodes its tensor map (driver entry point).
-cudaError_t en_job(EnJob *out, const Dims &d, const SplitLayout &L, const void *ws, const Inputs &in, const Work &w,
+[[nodiscard]] cudaError_t en_job(EnJob *out, const Dims &d, const SplitLayout &L, const void *ws, const Inputs &in, const Work &w,
                    int t0, int nt);
 // W-term launches per block of triplets: one per F, in the order gsel = 0, 1, 2.
 constexpr int SPLIT_WT_LAUNCHES = 3;
 // One block of triplets: the three W-term launches, then the energy launch,
 // on st.  w0 / w1 (optional) are recorded around the W-term launches.
-cudaError_t launch_split_block(WtBatch &wb, EnBatch &eb, int S, int num_sms, cudaStream_t st,
+[[nodiscard]] cudaError_t launch_split_block(WtBatch &wb, EnBatch &eb, int S, int num_sms, cudaStream_t st,
                                cudaEvent_t w0 = nullptr, cudaEvent_t w1 = nullptr);
 // Prepare the batches as launch_split_block would and fill the kernel-node
 // parameters of its launches: wb[0] is filled by the caller and copied into
 // wb[1], wb[2] (gsel 1, 2); wargs[f] / wp[f] belong to wb[f] (f < 3), eargs[0]
 // / ep to eb.  The nodes must run in the order wp[0], wp[1], wp[2], ep.
-cudaError_t split_block_params(WtBatch *wb, EnBatch &eb, int S, int num_sms, void **wargs, void **eargs,
+[[nodiscard]] cudaError_t split_block_params(WtBatch *wb, EnBatch &eb, int S, int num_sms, void **wargs, void **eargs,
                                cudaKernelNodeParams *wp, cudaKernelNodeParams *ep);
 
 // ---------------------------------------------------------------- FP64 path on the tensor cores (tc_rns.cu)
@@ -256,16 +257,16 @@ RnsTables rns_tables(int o, const int4 *trip, int n);
 // else those t.need marks).  *flag (device) is set to 1 when the inputs leave
 // the range of the integer grid: the results are then not to be used.  t must
 // stay alive until st reaches the copies' end.
-cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, const RnsTables &t, bool all, int *flag,
+[[nodiscard]] cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, const RnsTables &t, bool all, int *flag,
                             cudaStream_t st);
 int rns_prep_launches(int o, int v);
 // Jobs of triplets [t0, t0 + nt) for the two GEMM launches and the energy launch.
 void rns_block(const RnsLayout &L, void *ws, const Dims &d, const Inputs &in, const Work &w, const RnsTables &t, int t0,
                int nt, RnJob *j0, RnJob *j1, RnEnJob *en);
-cudaError_t launch_rns_block(RnBatch *gb, RnEnBatch &eb, int num_sms, cudaStream_t st, cudaEvent_t w0 = nullptr,
+[[nodiscard]] cudaError_t launch_rns_block(RnBatch *gb, RnEnBatch &eb, int num_sms, cudaStream_t st, cudaEvent_t w0 = nullptr,
                              cudaEvent_t w1 = nullptr);
 // As split_block_params: gp[0], gp[1], ep must run in this order.
-cudaError_t rns_block_params(RnBatch *gb, RnEnBatch &eb, int num_sms, void **gargs, void **eargs,
+[[nodiscard]] cudaError_t rns_block_params(RnBatch *gb, RnEnBatch &eb, int num_sms, void **gargs, void **eargs,
                              cudaKernelNodeParams *gp, cudaKernelNodeParams *ep);
 
 // Fill in the fields by which the reduction lists the weak triplets: those whose
@@ -280,7 +281,7 @@ void rns_weak(const RnsLayout &L, void *ws, RedJob *j);
 // bytes.  *digits receives the number of base-256 digits the factors needed
 // (at most 7); the call synchronises st once to read it.
 size_t df_scratch_bytes(int o, int v, int nq);
-cudaError_t df_assemble(const double *B, int nq, int o, int v, double *ovvv, double *ovoo, double *ovov,
+[[nodiscard]] cudaError_t df_assemble(const double *B, int nq, int o, int v, double *ovvv, double *ovoo, double *ovov,
                         void *scratch, int num_sms, cudaStream_t st, int *digits);
 // Device error flag of the assembly's kernels inside its scratch (0 = fine).
 int *df_error_flag(void *scratch, int o, int v, int nq);
@@ -302,6 +303,6 @@ struct RedBatch {
   int njobs;
   RedJob job[MAX_BATCH];
 };
-cudaError_t launch_reduce(const RedBatch &b, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_reduce(const RedBatch &b, cudaStream_t st);
 
 }  // namespace tc

@@ -229,6 +229,7 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
     cv_admit.notify_all();
     return;
   }
+  auto ok = [&e](cudaError_t x) { if (e == cudaSuccess) e = x; };   // the first failure of the preparation
   if (!q.dev_inputs) {
     const size_t O = q.o, V = q.v;
     const size_t n[6] = {O + V, O * V, O * O * V * V, O * V * V * V, O * V * O * O, O * V * O * V};
@@ -237,7 +238,7 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
     for (int a = 0; a < narr; ++a) {
       double *dst = (double *)(q.mem + off);
       const size_t cnt = (q.nq > 0 && a == 3) ? q.host[3].size() : n[a];
-      cudaMemcpyAsync(dst, q.host[a].data(), cnt * sizeof(double), cudaMemcpyHostToDevice, q.st);
+      ok(cudaMemcpyAsync(dst, q.host[a].data(), cnt * sizeof(double), cudaMemcpyHostToDevice, q.st));
       if (q.nq > 0 && a == 3) q.dB = dst;
       else q.din[a] = dst;
       off += cnt * sizeof(double);
@@ -248,7 +249,8 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
     const size_t O = q.o, V = q.v;
     double *ovvv = (double *)(q.mem + q.off_ints), *ovoo = ovvv + O * V * V * V, *ovov = ovoo + O * V * O * O;
     int digits = 0;
-    e = df_assemble(q.dB, q.nq, q.o, q.v, ovvv, ovoo, ovov, q.mem + q.off_df, ctx->num_sms, q.st, &digits);
+    if (e == cudaSuccess)
+      e = df_assemble(q.dB, q.nq, q.o, q.v, ovvv, ovoo, ovov, q.mem + q.off_df, ctx->num_sms, q.st, &digits);
     q.din[3] = ovvv;
     q.din[4] = ovoo;
     q.din[5] = ovov;
@@ -261,6 +263,7 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
       if (e == cudaSuccess && derr != 0) e = cudaErrorLaunchTimeout;
     }
     if (e != cudaSuccess) {
+      cudaStreamSynchronize(q.st);        // the copies read the job's host vectors
       std::lock_guard<std::mutex> lk(mu);
       for (auto &h : q.host) std::vector<double>().swap(h);
       fail_job(r, e == cudaErrorLaunchTimeout ? TC_ETIMEOUT : TC_ECUDA);
@@ -269,24 +272,24 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
   }
   char *base = q.mem + q.off_ws;
   const std::vector<int4> tab = plan::tables(q.d, q.L, nullptr);
-  cudaMemcpyAsync(base + q.L.trip, tab.data(), tab.size() * sizeof(int4), cudaMemcpyHostToDevice, q.st);
+  ok(cudaMemcpyAsync(base + q.L.trip, tab.data(), tab.size() * sizeof(int4), cudaMemcpyHostToDevice, q.st));
   q.w.trip = (const int4 *)(base + q.L.trip);
   q.w.orb = (const int4 *)(base + q.L.orb);
   q.w.partial = (double *)(base + q.L.partial);
   q.w.counter = (unsigned *)(base + q.L.counter);
   q.w.err = (int *)(base + q.L.counter + sizeof(unsigned));
-  cudaMemsetAsync(q.w.counter, 0, 3 * sizeof(unsigned), q.st);
+  ok(cudaMemsetAsync(q.w.counter, 0, 3 * sizeof(unsigned), q.st));
   const Inputs in{q.din[0], q.din[1], q.din[2], q.din[3], q.din[4], q.din[5]};
   int out_of_range = 0;
   if (split) {
-    launch_split_prep(q.SL, in, q.mem + q.off_split, q.st);
+    ok(launch_split_prep(q.SL, in, q.mem + q.off_split, q.st));
   } else if (q.group == G_RNS) {
     q.rt = rns_tables(q.o, tab.data(), q.d.n_trip);
-    launch_rns_prep(q.RL, in, q.mem + q.off_split, q.rt, true, q.w.err + 1, q.st);
-    cudaMemcpyAsync(&out_of_range, q.w.err + 1, sizeof(int), cudaMemcpyDeviceToHost, q.st);
+    ok(launch_rns_prep(q.RL, in, q.mem + q.off_split, q.rt, true, q.w.err + 1, q.st));
+    ok(cudaMemcpyAsync(&out_of_range, q.w.err + 1, sizeof(int), cudaMemcpyDeviceToHost, q.st));
   }
-  cudaEventRecord(q.ready, q.st);
-  e = cudaStreamSynchronize(q.st);        // the copies read the job's host vectors
+  ok(cudaEventRecord(q.ready, q.st));
+  ok(cudaStreamSynchronize(q.st));        // the copies read the job's host vectors
   std::lock_guard<std::mutex> lk(mu);
   if (out_of_range) {                     // beyond the integer grid: the DMMA kernel
     q.group = 0;
@@ -414,7 +417,11 @@ bool Server::run_iteration(int g, std::vector<std::shared_ptr<Req>> &jobs) {
     }
     if (e == cudaSuccess) e = split_block_params(wb, eb, g + 1, ctx->num_sms, args, eargs, kp, &ep);
   }
-  if (e != cudaSuccess) return false;
+  if (e != cudaSuccess) {
+    std::lock_guard<std::mutex> lk(mu);
+    for (auto &r : jobs) fail_job(r, TC_ECUDA);
+    return false;
+  }
   if (!exec[g]) {
     // the group's graph: FP64, [zero the work counter] -> [multi-job kernel];
     // split, [W-term F0] -> [F1] -> [F2] -> [energy]; FP64 on the tensor
