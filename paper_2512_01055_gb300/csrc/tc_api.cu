@@ -148,7 +148,7 @@ tc_status run_device(tc_ctx *ctx, int o, int v, const tc::Inputs &in, int prec, 
   w.err = (int *)(base + L.counter + sizeof(unsigned));
   double *e_trip = (double *)(base + L.e_trip);
   double *dout = (double *)(base + L.out);
-  TC_CUDA(ctx, cudaMemsetAsync(w.counter, 0, 3 * sizeof(unsigned), st));
+  TC_CUDA(ctx, cudaMemsetAsync(w.counter, 0, tc::plan::COUNTER_WORDS * sizeof(unsigned), st));
   tc::RnsTables rt;
   if (e_ijk_dev) TC_CUDA(ctx, cudaMemsetAsync(e_ijk_dev, 0, sizeof(double) * (size_t)o * o * o, st));
   int launches = d.n_trip > 0 ? 2 : 1;                   // the reduction

@@ -32,6 +32,8 @@ inline Dims make_dims(int o, int v, int nt, int n_trip_override = -1, int min_op
   return d;
 }
 
+constexpr int COUNTER_WORDS = 3;   // work counter, then Work::err[2]
+
 struct Layout {            // byte offsets inside a job's workspace
   size_t trip, orb, partial, e_trip, out, counter, total;
 };
@@ -44,7 +46,7 @@ inline Layout make_layout(const Dims &d) {
   L.partial = off; off = align256(off + 2 * sizeof(double) * (size_t)std::max<long long>(1, d.n_items));
   L.e_trip = off;  off = align256(off + sizeof(double) * (size_t)std::max(1, d.n_trip));
   L.out = off;     off = align256(off + 4 * sizeof(double));
-  L.counter = off; off = align256(off + 2 * sizeof(unsigned));
+  L.counter = off; off = align256(off + COUNTER_WORDS * sizeof(unsigned));
   L.total = off;
   return L;
 }

@@ -278,7 +278,7 @@ void Server::start_prep(const std::shared_ptr<Req> &r) {
   q.w.partial = (double *)(base + q.L.partial);
   q.w.counter = (unsigned *)(base + q.L.counter);
   q.w.err = (int *)(base + q.L.counter + sizeof(unsigned));
-  ok(cudaMemsetAsync(q.w.counter, 0, 3 * sizeof(unsigned), q.st));
+  ok(cudaMemsetAsync(q.w.counter, 0, plan::COUNTER_WORDS * sizeof(unsigned), q.st));
   const Inputs in{q.din[0], q.din[1], q.din[2], q.din[3], q.din[4], q.din[5]};
   int out_of_range = 0;
   if (split) {
