@@ -1065,20 +1065,6 @@ rns_gemm_kernel(const __grid_constant__ RnBatch B) {
 constexpr int WX = 73, WY = 9;               // W block index = x WX + y WY + z (8-byte words)
 constexpr int WBLK = 7 * WX + 7 * WY + 8;
 
-// 1 / x for |x| in [2^-500, 2^500]: the hardware's approximation r (about 20
-// bits) and one third-order step r (1 + e + e^2), e = 1 - x r, whose error e^3
-// is below the last place.  Three FP64 operations where a division takes ten.
-__device__ __forceinline__ double rcp_fast(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-__device__ __forceinline__ double recip(double x) {
-  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7FF;
-  return ex - 523u <= 1000u ? rcp_fast(x) : 1.0 / x;
-}
-
 // |x| as a float (its leading 20 bits; beyond the float range 0 or infinity),
 // without the FP64 pipe.
 __device__ __forceinline__ float abs_float(double x) {
@@ -1106,7 +1092,9 @@ __device__ __forceinline__ double u128_double(unsigned __int128 x) {
 // |W| < 2^59 units (14 standard deviations on data of uniform size; larger
 // values take the same formulas in FP64), converted once each.  Then
 // sum_s w_s br_s = (sum_s br_s^2) / 3 - 6 d^2, formed in 128-bit integers (the
-// integer pipes have room beside the FP64 pipe); 37 FP64 operations a point in all.
+// integer pipes have room beside the FP64 pipe); 34 FP64 operations a point and the
+// division by D, which is left to the compiler: an own reciprocal of three
+// operations made o=12 v=132 1.4 % faster and was right to the last place only.
 // The weak triplets' bound, WEAK_N4 times the sum of |1/D|, is summed in FP32.
 // Five small CTAs on an SM keep the pipe fed while one of them loads.
 // Orbits with equal tiles list their canonical points (36 x 8 of 512 points for
@@ -1265,7 +1253,7 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
           const double vs = fma(T(0, p0), G(0, p1, p2), fma(T(1, p1), G(1, p0, p2), T(2, p2) * G(2, p0, p1)));
           n5 = s == 0 ? vs * br[0] : fma(vs, br[s], n5);
         }
-        double r = recip(Eab[l3[0] * NT + l3[1]] - __ldg(J.eps + o + gc));
+        double r = 1.0 / (Eab[l3[0] * NT + l3[1]] - __ldg(J.eps + o + gc));
         if (ga == gb || gb == gc) r *= ga == gc ? 1.0 / 6.0 : 0.5;   // the point's share of the bracket sums
         const int dS = S0 - sexp - __ldg(J.ev + ga) - __ldg(J.ev + gb) - __ldg(J.ev + gc);
         if (dS != 0) {
