@@ -6,7 +6,7 @@
 //
 // Slices.  Every FP64 operand x is written as s BF16 numbers x_0 + ... + x_{s-1}
 // with x_0 = bf16(x) and x_p = bf16(x - x_0 - ... - x_{p-1}) (round to
-// nearest; the FP64 residual is exact), the splitting used to emulate higher
+// nearest; the residuals exact, tc_slices.cuh), the splitting used to emulate higher
 // precision with BF16 products (Henry, Tang, Heinecke, ARITH 2019).  A product
 // is approximated by the slice pairs (p, q) with p + q < s.
 //
@@ -67,6 +67,7 @@
 
 #include "tc_internal.cuh"
 #include "tc_ptx.cuh"
+#include "tc_slices.cuh"
 
 namespace tc {
 namespace {
@@ -962,34 +963,16 @@ tc_energy_kernel(const __grid_constant__ EnBatch B) {
 //   hb   B  [r][q][nc][ho]    row z,      K l:  -(r z | q l)           = -ovoo[r][z][q][l]
 // Every image is ordered by the first occupied index of the tensor it reads.
 
-// The slices of 8 values, BF16, written to out + p step (and outT + p step) for
-// p < S.  x becomes a float pair (h, l) once, l rounded to odd (its last bit set
-// when bits are lost), so later roundings to fewer bits come out as from x
-// itself (Boldo and Melquiond): four FP64 operations, GB300's FP64 pipe being
-// 1/64 of its FP32 pipe, where taking every slice and residual in FP64 costs
-// three each.  A slice is the BF16 nearest to h + l: of their FP32 sum s, or
-// where s lies midway between two, of the side its rounding error (TwoSum)
-// points to; s minus the slice, exact, and that error are the next pair.
+// The slices of 8 values (tc_slices.cuh), written to out + p step (and outT + p
+// step) for p < S.
 __device__ __forceinline__ void write_slices(const double (&x)[8], int S, uint4 *out, uint4 *outT, size_t step) {
-  float h[8], l[8];
+  Slicer a[8];
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    h[u] = __double2float_rn(x[u]);
-    const double r = x[u] - (double)h[u];
-    l[u] = __double2float_rz(r);
-    if (__double2loint(r) & 0x1FFFFFFF) l[u] = __uint_as_float(__float_as_uint(l[u]) | 1u);
-  }
+  for (int u = 0; u < 8; ++u) a[u] = slicer(x[u]);
   for (int p = 0; p < S; ++p) {
     uint32_t b[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const float s = h[u] + l[u], t = s - h[u], er = (h[u] - (s - t)) + (l[u] - t);
-      const uint32_t bits = __float_as_uint(s);
-      b[u] = __bfloat16_as_ushort(__float2bfloat16_rn(s));
-      if ((bits & 0xFFFF) == 0x8000 && er != 0.f) b[u] = (bits >> 16) + (((__float_as_uint(er) ^ bits) >> 31) ^ 1u);
-      h[u] = s - __uint_as_float(b[u] << 16);
-      l[u] = er;
-    }
+    for (int u = 0; u < 8; ++u) b[u] = next_slice(a[u], p);
     const uint4 q = make_uint4(b[0] | b[1] << 16, b[2] | b[3] << 16, b[4] | b[5] << 16, b[6] | b[7] << 16);
     out[p * step] = q;
     if (outT) outT[p * step] = q;
