@@ -148,3 +148,15 @@ def test_inputs_beyond_the_grid_do_not_run_the_residue_products():
     print(f"good {good.seconds:.4f} s, of it residue kernels {good.kernel_seconds:.4f} s; "
           f"beside the DMMA kernel {bad.seconds - bad.kernel_seconds:.4f} s")
     assert bad.seconds - bad.kernel_seconds < 0.5 * good.kernel_seconds
+
+
+# o = 2, v = 9: the smallest shape of the residues; v = 8, o = 1 and K beyond 1024 take the DMMA kernel
+@pytest.mark.parametrize("o,v,residues", [(2, 9, True), (2, 8, False), (1, 12, False), (3, 9, True), (9, 10, True),
+                                          (2, 504, True), (2, 505, False)])
+def test_which_kernel_runs(o, v, residues):
+    d = _random(o, v, 900 + v)
+    r, e = _energy(o, v, d)
+    assert (r.prep_seconds > 0.0) == residues and (r.wterm_seconds < r.kernel_seconds) == residues
+    e_ref, ref = _noalloc(o, v, d)
+    assert np.abs(e - ref).max() <= 1e-12 * np.abs(ref).max()
+    assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
