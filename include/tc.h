@@ -59,9 +59,9 @@ typedef enum {
 typedef enum {
   TC_FP64 = 0,         /* FP64-accurate W, FP64 epilogue and sums.  W as exact integer products in residues on
                           the BF16 tensor cores: operands rounded once to one power-of-two grid per array (refined
-                          for orbitals that are weak in every array), W to 64 bits.  W of a triplet is within about
-                          2^-50 of its root mean square, as FP64 accumulation leaves it; triplets too weak for that
-                          on the common grid are formed again with FP64 tensor-core (DMMA) tiles.  Everything runs
+                          for orbitals that are weak in every array), W to 64 bits.  W of a triplet is within 2^-49
+                          of its root mean square, mostly 2^-51 as FP64 accumulation leaves it; triplets too weak for
+                          that on the common grid are formed again with FP64 tensor-core (DMMA) tiles.  Everything runs
                           on DMMA tiles where the shape (o < 2, v < 9, K = 2v + 2o padded above 1024), the memory
                           (budget and device) or the inputs (infinities, NaN, an array's largest norm outside
                           2^+-100) do not allow residues; the two agree to the accuracy stated, not to the bit */

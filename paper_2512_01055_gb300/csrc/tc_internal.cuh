@@ -194,7 +194,7 @@ struct RnsGeom {
 // the weak triplets' bound and the list of weak triplets, mask of occupied pairs.
 struct RnsLayout {
   RnsGeom g;
-  size_t pa, pa2, hc, hc2, tb, hb, y, ra, rt, rb, rh, mx, ex, unit, margin, weak, need;
+  size_t pa, pa2, hc, hc2, tb, hb, y, ra, rt, rb, rh, mx, nz, ex, unit, margin, weak, need;
   size_t total;
 };
 // Host tables of a triplet list.  A unit is one F GEMM of one triplet:
@@ -231,6 +231,7 @@ struct RnEnJob {         // one job's block of triplets in an energy launch
   const double *eps, *t1, *ovov;
   const long long *y;
   const int *ev, *uo, *sh;
+  const double *nz;      // W's squared error (Scales::nz)
   double *partial;       // [n_items][2], slot t * items_per_trip + chunk
   double *margin;        // [n_items]: |E[4]_ST| of the item less the weak triplets' bound
   int t0, nt;

@@ -26,11 +26,11 @@
 // Scales.  W_ijk^abc is a sum of products with one fixed-point grid,
 // 2^-(e_a + e_b + e_c + u_i + u_j + u_k + SS): an exponent >= 0 per virtual and
 // per occupied orbital from the norms of integrals and amplitudes together, and
-// a global shift from the largest norms.  The exponents raise no row above the
-// largest of its array, so they refine the grid of weak orbitals and coarsen
-// none.  The contributions of all six permutations are integers on one grid:
-// they are added by 64-bit integer reductions in L2, which are exact and free
-// of order.
+// a global shift from the largest scaled norms.  The exponents raise no row by
+// more than 2 bits over the largest of its array: they refine the grid of weak
+// orbitals and hardly coarsen that of the others.  The contributions of all six
+// permutations are integers on one grid: they are added by 64-bit integer
+// reductions in L2, which are exact and free of order.
 //
 // W as three GEMMs per triplet (F(p,q,r) of tc_split.cu, the same operand
 // segments):  W_abc = F(i,j,k)[ab,c] + F(i,k,j)[ac,b] + F(j,k,i)[bc,a].
@@ -56,8 +56,11 @@
 // accumulation keeps them relative to each product.  The energy kernel therefore
 // sums, beside E[4]_ST, what E[4]_ST would be if W had WEAK_RMS units of its
 // 64-bit fraction everywhere, and the DMMA kernel forms the triplets below that
-// again.
-#include <algorithm>
+// accumulation keeps them relative to each product.  The rounding error of a
+// triplet's W follows from the norms of its rows.  The energy kernel sums, beside
+// E[4]_ST, what E[4]_ST would be if W were 2^49 times that error everywhere, and
+// the DMMA kernel forms the triplets below that again.
+
 #include <type_traits>
 
 #include "tc_internal.cuh"
@@ -96,14 +99,15 @@ constexpr int SMEM_DYN_MAX = 232448 - 2048;
 constexpr int NT = 8;                        // tile edge of the energy orbits
 constexpr int NT2 = NT * NT, NT3 = NT2 * NT;
 constexpr int EN_THREADS = 128, EN_CTAS = 5;   // per CTA, CTAs per SM
-// W is off by about 2^2.4 units where the operands have full-size norms, and on
-// data of uniform size its rms is above 2^53 units (2^57 and 2^56 per operand norm
-// less a bit each for powers of two, over sqrt(K); no triplet below 2^53 in 50
-// shapes from o=2 v=9 to o=2 v=504 and o=6 v=290): 2^-51 to 2^-53 of it, as the
-// DMMA kernel's.  WEAK_RMS is the least rms the residues are trusted with, an
-// error of 2^-49.6.  The bracket sum n4 of independent W of variance 1 has mean 72.
-constexpr double WEAK_RMS = 0x1p52;
-constexpr double WEAK_N4 = 72.0 * WEAK_RMS * WEAK_RMS;
+// A triplet's W has to be 2^49 times its error in the root mean square.  The bound
+// of the error takes every row at its largest, 1 to 2 bits over what it is: with
+// factors of 2^-9 to 1 per orbital, triplets at that edge among them, energies are
+// as far from 80-bit references as the DMMA kernel's (at most 1.0e-15 and 9.7e-16
+// of |E[4]| + |V r3(W) / D|), whose W is right to 2^-51.2 (K = 132) to 2^-50.4
+// (K = 400).  On data of uniform size W is above 2^52 times the bound (50 shapes
+// from o=2 v=9 to o=2 v=504 and o=6 v=290).  The bracket sum n4 of independent W
+// of variance 1 has mean 72.
+constexpr double WEAK_N4 = 72.0 * 0x1p98;
 
 constexpr int ERR_TIMEOUT_FULL = 11, ERR_TIMEOUT_EMPTY = 12, ERR_TIMEOUT_ACCFULL = 13,
               ERR_TIMEOUT_ACCEMPTY = 14, ERR_TIMEOUT_TEARDOWN = 15;
@@ -203,6 +207,10 @@ struct Scales {
   int *fv, *fu;                    // [v], [o]: share of them, in 256ths, that suits every row
   int *ev, *uo;                    // [v], [o]: the exponents taken
   int *sh;                         // [5]: shifts of the four operands and SS; sh[5]: 1 if any of dv, du is not 0
+  unsigned long long *pm, *qm;     // with exponents, [2][o]: largest scaled squared norm of arrays 0, 1 by p; [2][o][o]: of
+                                   // arrays 2, 3 by (r, q)
+  double *nz;                      // squared error of W in units of its fraction: [0] of any triplet without exponents;
+                                   // with them [1 + p] and [1 + o + r o + q], summed over a triplet's p and (r, q)
   int *flag;                       // 1: inputs out of the range the integer grid covers
 };
 
@@ -296,13 +304,13 @@ __global__ void rns_norms(Inputs in, int o, int v, Scales s) {
 // scaling an input array by a power of two changes none of them).  d of an
 // orbital is the least slack of the rows that hold it, over all four arrays: 0
 // where any array has a row of full size.  A row holds three orbitals, so the
-// sum of their d may exceed its slack; each orbital then takes the share
-// slack / sum of its d, the smallest over its rows, which keeps every row
-// within the array's largest.  (Where all arrays carry one factor per orbital,
-// the shares stay near 1 and the exponents take it out.  An exponent from the
-// integrals alone, used before, scaled amplitudes up with it: W lost all digits
-// when one orbital's ovvv was 2^-24 of the others'.)
-constexpr int D_MAX = 16;
+// sum of their d may exceed its slack; each orbital then takes the share (slack +
+// SPARE) / sum of its d, the smallest over its rows, which keeps every row within
+// 2^SPARE of the array's largest.  Where all arrays carry one factor per orbital,
+// the shares stay 1 and the exponents take it out (SPARE = 0: some row's scatter
+// halves them).  An exponent from the integrals alone scales amplitudes up with
+// it: W lost all digits when one orbital's ovvv was 2^-24 of the others'.
+constexpr int D_MAX = 16, SPARE = 2;
 constexpr int NO_ROW = 1 << 20;                           // slack of a row of zeros
 
 // Slack of a squared norm (IEEE bits) against the array's largest.
@@ -353,7 +361,7 @@ __device__ void shares(int o, int v, const Scales &s) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, st = (long long)gridDim.x * blockDim.x;
   auto row = [&](double n, int k, const int *d0, const int *d1, const int *d2, int *f0, int *f1, int *f2) {
     const int sum = __ldcg(d0) + __ldcg(d1) + __ldcg(d2);
-    const int sl = slack((unsigned long long)__double_as_longlong(n), expo(mb[k]));
+    const int sl = slack((unsigned long long)__double_as_longlong(n), expo(mb[k])) + SPARE;
     if (sl >= sum) return;
     const int f = 256 * sl / sum;
     int *const ff[3] = {f0, f1, f2};
@@ -373,10 +381,76 @@ __device__ void shares(int o, int v, const Scales &s) {
   }
 }
 
+__device__ __forceinline__ int taken(const int *d, const int *f, int x) { return __ldcg(d + x) * __ldcg(f + x) >> 8; }
+__device__ __forceinline__ double pow4(int e) { return __longlong_as_double((long long)(1023 + 2 * e) << 52); }   // |e| <= 500
+
+// Largest scaled squared norms by p (arrays 0, 1; a warp takes the rows of one
+// (p, x)) and by (r, q) (arrays 2, 3; a warp per pair).
+__device__ void scaled_max(int o, int v, const Scales &s) {
+  if (__ldcg(s.sh + 5) == 0) return;
+  const int lane = threadIdx.x & 31, w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int warps = gridDim.x * (blockDim.x >> 5);
+  auto bits = [](double n, int e) { return (unsigned long long)__double_as_longlong(n * pow4(e)); };
+  auto top = [](unsigned long long b) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, off));
+    return b;
+  };
+  for (int w = w0; w < o * v; w += warps) {
+    const int p = w / v, e0 = taken(s.du, s.fu, p) + taken(s.dv, s.fv, w % v);
+    unsigned long long b0 = 0, b1 = 0;
+    for (int y = lane; y < v; y += 32) {
+      const int e = e0 + taken(s.dv, s.fv, y);
+      b0 = max(b0, bits(s.ra[(long long)w * v + y], e));
+      b1 = max(b1, bits(s.rt[(long long)w * v + y], e));
+    }
+    b0 = top(b0);
+    b1 = top(b1);
+    if (lane == 0) {
+      if (b0 > *(volatile unsigned long long *)(s.pm + p)) atomicMax(s.pm + p, b0);
+      if (b1 > *(volatile unsigned long long *)(s.pm + o + p)) atomicMax(s.pm + o + p, b1);
+    }
+  }
+  for (int w = w0; w < o * o; w += warps) {
+    const int r = w / o, q = w % o, e0 = taken(s.du, s.fu, r) + taken(s.du, s.fu, q);
+    unsigned long long b2 = 0, b3 = 0;
+    for (int z = lane; z < v; z += 32) {
+      const int e = e0 + taken(s.dv, s.fv, z);
+      b2 = max(b2, bits(s.rb[(long long)w * v + z], e));
+      b3 = max(b3, bits(s.rh[((long long)r * v + z) * o + q], e));
+    }
+    b2 = top(b2);
+    b3 = top(b3);
+    if (lane == 0) {
+      s.qm[w] = b2;
+      s.qm[o * o + w] = b3;
+    }
+  }
+}
+
 // The exponents taken.
 __device__ void take_exps(int o, int v, const Scales &s) {
-  for (int x = threadIdx.x; x < v; x += blockDim.x) s.ev[x] = s.dv[x] * __ldcg(s.fv + x) >> 8;
-  for (int p = threadIdx.x; p < o; p += blockDim.x) s.uo[p] = s.du[p] * __ldcg(s.fu + p) >> 8;
+  for (int x = threadIdx.x; x < v; x += blockDim.x) s.ev[x] = taken(s.dv, s.fv, x);
+  for (int p = threadIdx.x; p < o; p += blockDim.x) s.uo[p] = taken(s.du, s.fu, p);
+}
+
+// Each array's largest scaled squared norm (IEEE bits), to every thread of the CTA.
+__device__ void array_scaled_max(int o, int v, const Scales &s, unsigned long long (&mb)[4]) {
+  if (__ldcg(s.sh + 5) == 0) {
+    array_max(v, s, mb);
+    return;
+  }
+  __shared__ unsigned long long m[4];
+  if (threadIdx.x < 4) m[threadIdx.x] = 0;
+  __syncthreads();
+  for (int x = threadIdx.x; x < 2 * (o + o * o); x += blockDim.x) {
+    const unsigned long long b = __ldcg(x < 2 * o ? s.pm + x : s.qm + (x - 2 * o));
+    unsigned long long *const k = m + (x < 2 * o ? x / o : 2 + (x - 2 * o) / (o * o));
+    if (b > *(volatile unsigned long long *)k) atomicMax(k, b);
+  }
+  __syncthreads();
+  for (int k = 0; k < 4; ++k) mb[k] = m[k];
+  __syncthreads();
 }
 
 // Shifts of the four operands (one CTA).  A row of norm n is scaled to at
@@ -384,11 +458,9 @@ __device__ void take_exps(int o, int v, const Scales &s) {
 // share the grid (sa + sb = sah + sbh = SS); the pair with room to spare is
 // scaled down.  Arrays of zeros take shift 0; inputs whose norms leave
 // [2^-100, 2^100] or are not finite set the flag.
-__device__ void shifts(int v, const Scales &s) {
-  unsigned long long mb[4];
+__device__ void shifts(const Scales &s, const unsigned long long (&mb)[4]) {
   int i[4];
   bool any[4];
-  array_max(v, s, mb);
   if (threadIdx.x != 0) return;
   for (int k = 0; k < 4; ++k) {
     any[k] = mb[k] != 0;
@@ -415,23 +487,54 @@ __device__ void shifts(int v, const Scales &s) {
   s.sh[4] = sa + sb;
 }
 
-__global__ void rns_wanted(int o, int v, Scales s) { wanted(o, v, s); }
-__global__ void rns_shares(int o, int v, Scales s) { shares(o, v, s); }
-__global__ void rns_scales(int o, int v, Scales s) {
-  take_exps(o, v, s);
-  shifts(v, s);
+// W's squared error, from the rounding of the operands to the grid: an element of
+// a row is off by a variance of 1/12, a product by (|a|^2 + |b|^2) / 12 in units
+// of the grid, C_P of which make a unit of W's fraction; 1 more for each of the
+// three F's own fraction (one CTA).
+__device__ void noise(int o, const Scales &s, const unsigned long long (&mb)[4]) {
+  auto scaled = [&](unsigned long long b, int k) {
+    return __longlong_as_double((long long)b) * pow4(s.sh[k]) * (1.0 / (12.0 * C_P * C_P));
+  };
+  if (threadIdx.x == 0) {
+    double n = 0.0;
+    for (int k = 0; k < 4; ++k) n += scaled(mb[k], k);
+    s.nz[0] = 6.0 * n + 3.0;
+  }
+  if (s.sh[5] == 0) return;
+  for (int p = threadIdx.x; p < o; p += blockDim.x)
+    s.nz[1 + p] = 2.0 * (scaled(__ldcg(s.pm + p), 0) + scaled(__ldcg(s.pm + o + p), 1));
+  for (int w = threadIdx.x; w < o * o; w += blockDim.x)
+    s.nz[1 + o + w] = scaled(__ldcg(s.qm + w), 2) + scaled(__ldcg(s.qm + o * o + w), 3);
 }
 
-// All three steps by one CTA, for jobs where their launches take longer than
+// The last step, by one CTA: exponents, shifts, errors.
+__device__ void finish_scales(int o, int v, const Scales &s) {
+  unsigned long long mb[4];
+  take_exps(o, v, s);
+  array_scaled_max(o, v, s, mb);
+  shifts(s, mb);
+  __syncthreads();
+  noise(o, s, mb);
+}
+
+__global__ void rns_wanted(int o, int v, Scales s) { wanted(o, v, s); }
+__global__ void rns_shares(int o, int v, Scales s) { shares(o, v, s); }
+__global__ void rns_scaled_max(int o, int v, Scales s) { scaled_max(o, v, s); }
+__global__ void rns_scales(int o, int v, Scales s) { finish_scales(o, v, s); }
+
+// All four steps by one CTA, for jobs where their launches take longer than
 // their work: up to SCALES_ONE rows of ovvv.
+// (Preparation, all steps in one launch against four: o=6 v=36 39 / 45 us, o=9 v=77
+// 153 / 160; where there are exponents 53 / 53 and 214 / 167, o=8 v=104 312 / 235.)
 constexpr long long SCALES_ONE = 1 << 16;
 __global__ void __launch_bounds__(1024) rns_scales_one(int o, int v, Scales s) {
   wanted(o, v, s);
   __syncthreads();
   shares(o, v, s);
   __syncthreads();
-  take_exps(o, v, s);
-  shifts(v, s);
+  scaled_max(o, v, s);
+  __syncthreads();
+  finish_scales(o, v, s);
 }
 
 // ---------------------------------------------------------------- operand images
@@ -1095,7 +1198,8 @@ __device__ __forceinline__ double u128_double(unsigned __int128 x) {
 // integer pipes have room beside the FP64 pipe); 34 FP64 operations a point and the
 // division by D, which is left to the compiler: an own reciprocal of three
 // operations made o=12 v=132 1.4 % faster and was right to the last place only.
-// The weak triplets' bound, WEAK_N4 times the sum of |1/D|, is summed in FP32.
+// The weak triplets' bound, the sum of |1/D| (times WEAK_N4 and W's squared error
+// at the end), is summed in FP32.
 // Five small CTAs on an SM keep the pipe fed while one of them loads.
 // Orbits with equal tiles list their canonical points (36 x 8 of 512 points for
 // two equal tiles, 120 for three), so no warp runs for points outside them.
@@ -1281,7 +1385,14 @@ rns_energy_kernel(const __grid_constant__ RnEnBatch B) {
       double e4 = 0.0, e5 = 0.0, er = 0.0;
       for (int k = 0; k < EN_THREADS / 32; ++k) { e4 += s_red[k][0]; e5 += s_red[k][1]; er += s_abs[k]; }
       const double f = __longlong_as_double((long long)(1023 - sprev) << 52);
-      er = (fabs(e4) - WEAK_N4 * er) * f * (C_P * C_P / 3.0) * f;
+      double nz = J.nz[0];
+      if (J.sh[5]) {
+        const double *np = J.nz + 1, *nq = np + o;
+        auto pair = [&](int r, int q) { return nq[r * o + q] + nq[q * o + r]; };
+        nz = 3.0 + (np[occ[0]] + np[occ[1]] + np[occ[2]]) +
+             (pair(occ[0], occ[1]) + pair(occ[0], occ[2]) + pair(occ[1], occ[2]));
+      }
+      er = (fabs(e4) - WEAK_N4 * nz * er) * f * (C_P * C_P / 3.0) * f;
       e4 = e4 * f * (C_P * C_P / 3.0) * f;
       e5 = e5 * f * C_P;
       const long long idx = (long long)(J.t0 + tl) * d.items_per_trip + chunk;
@@ -1311,6 +1422,9 @@ Scales scales_at(const RnsLayout &L, void *ws, int *flag) {
   s.fv = s.du + o;
   s.fu = s.fv + v;
   s.sh = s.fu + o;
+  s.pm = s.no + 4 * o + 1;                               // behind the number of weak triplets
+  s.qm = s.pm + 2 * o;
+  s.nz = (double *)(b + L.nz);
   s.flag = flag;
   return s;
 }
@@ -1423,7 +1537,8 @@ RnsLayout rns_layout(const Dims &d) {
   L.rt = take(O * V * V * 8);
   L.rb = take(O * O * V * 8);
   L.rh = take(O * V * O * 8);
-  L.mx = take((4 * (V + O) + 1) * 8);
+  L.mx = take((4 * (V + O) + 1 + 2 * O + 2 * O * O) * 8);
+  L.nz = take((1 + O + O * O) * 8);
   L.ex = take((3 * (V + O) + 8) * 4);
   L.unit = take((size_t)3 * std::max(1, d.n_trip) * 4);
   L.margin = take((size_t)std::max<long long>(1, d.n_items) * 8);
@@ -1453,7 +1568,7 @@ RnsTables rns_tables(int o, const int4 *trip, int n) {
   return t;
 }
 
-int rns_prep_launches(int o, int v) { return (long long)o * v * v <= SCALES_ONE ? 3 : 5; }
+int rns_prep_launches(int o, int v) { return (long long)o * v * v <= SCALES_ONE ? 3 : 6; }
 
 cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, const RnsTables &t, bool all, int *flag,
                             cudaStream_t st) {
@@ -1462,8 +1577,8 @@ cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, cons
   const Scales s = scales_at(L, ws, flag);
   cudaError_t e = cudaMemcpyAsync(b + L.unit, t.unit.data(), t.unit.size() * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && !all) e = cudaMemcpyAsync(b + L.need, t.need.data(), t.need.size(), cudaMemcpyHostToDevice, st);
-  // the maxima and the number of weak triplets behind them
-  if (e == cudaSuccess) e = cudaMemsetAsync(b + L.mx, 0, (4 * ((size_t)g.v + g.o) + 1) * 8, st);
+  // the maxima per array and orbital, the number of weak triplets, the scaled maxima by p
+  if (e == cudaSuccess) e = cudaMemsetAsync(b + L.mx, 0, (4 * ((size_t)g.v + g.o) + 1 + 2 * (size_t)g.o) * 8, st);
   if (e != cudaSuccess) return e;
   const unsigned char *need = all ? nullptr : (const unsigned char *)(b + L.need);
   rns_norms<<<PREP_BLOCKS, PREP_THREADS, 4 * ((size_t)g.v + g.o) * 8, st>>>(in, g.o, g.v, s);
@@ -1472,6 +1587,7 @@ cudaError_t launch_rns_prep(const RnsLayout &L, const Inputs &in, void *ws, cons
   } else {
     rns_wanted<<<1, 512, 0, st>>>(g.o, g.v, s);
     rns_shares<<<152 * 2, 256, 0, st>>>(g.o, g.v, s);
+    rns_scaled_max<<<152 * 2, 256, 0, st>>>(g.o, g.v, s);
     rns_scales<<<1, 512, 0, st>>>(g.o, g.v, s);
   }
   unsigned char *ub = (unsigned char *)b;
@@ -1516,6 +1632,7 @@ void rns_block(const RnsLayout &L, void *ws, const Dims &d, const Inputs &in, co
   E.ev = s.ev;
   E.uo = s.uo;
   E.sh = s.sh;
+  E.nz = s.nz;
   E.partial = w.partial;
   E.margin = (double *)(b + L.margin);
   E.t0 = t0;

@@ -160,3 +160,26 @@ def test_which_kernel_runs(o, v, residues):
     e_ref, ref = _noalloc(o, v, d)
     assert np.abs(e - ref).max() <= 1e-12 * np.abs(ref).max()
     assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
+
+
+@pytest.mark.parametrize("spread", [3, 6, 9])
+def test_factors_per_orbital_keep_the_residues(spread):
+    """Every orbital's integrals and amplitudes times its own factor between 2^-spread and 1: the exponents take the
+    factors out, and no triplet needs the DMMA kernel (which would show in the number of launches)."""
+    import torch
+    o, v = 6, 40
+    d = _random(o, v, 78)
+    launches = _energy(o, v, d)[0].launches
+    g = torch.Generator(device="cuda").manual_seed(6)
+    fo, fv = (torch.exp2(-spread * torch.rand(n, generator=g, device="cuda", dtype=torch.float64)) for n in (o, v))
+    d["ovvv"] *= fo[:, None, None, None] * fv[None, :, None, None] * fv[None, None, :, None] * fv
+    d["ovoo"] *= fo[:, None, None, None] * fv[None, :, None, None] * fo[None, None, :, None] * fo
+    d["t2"] *= fo[:, None, None, None] * fo[None, :, None, None] * fv[None, None, :, None] * fv
+    r, e = _energy(o, v, d)
+    e_ref, ref = _noalloc(o, v, d)
+    nz = ref != 0.0
+    print(f"spread 2^-{spread}: {r.launches - launches} launches more, worst relative error of a triplet "
+          f"{np.abs(e[nz] / ref[nz] - 1).max():.2e}")
+    assert r.launches == launches
+    assert np.all(np.abs(e - ref) <= 1e-11 * np.abs(ref))
+    assert abs(r.e_t - e_ref) <= 1e-12 * np.abs(ref).sum()
