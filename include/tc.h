@@ -130,8 +130,9 @@ tc_status tc_init(tc_ctx **ctx, const tc_options *opt);
  * TC_SPLIT_BF16, <= 0 for the default; ignored for TC_FP64.  TC_FP64 holds
  * residue images of the operands (30 bytes per element of ovvv in each of two
  * orders) besides tc_workspace_bytes while the context's budget and the device
- * have room for them; they are given back after the call when they exceed a
- * quarter of the budget, and when another call needs the memory.
+ * have room for them beside the context's other buffers and served jobs; they
+ * are given back after the call when they exceed a quarter of the budget, and
+ * later when another call or a served job of the context needs the room.
  * e_ijk (optional, may be NULL): host array [o][o][o] that receives the
  * weighted contribution of each occupied triplet i >= j >= k at [i][j][k]
  * (E_(T) is their sum); entries with i < j or j < k are set to 0. */
@@ -246,7 +247,8 @@ tc_status tc_combine_parts(const double *parts, int n, double *e_t);
  * for a small job of its group that is being handed in or prepared), the slices
  * shared fairly, so a job submitted while others
  * run starts within an iteration and small jobs are not stuck behind large
- * ones.  A job's result does not depend on the other jobs it ran with.
+ * ones.  A job's result does not depend on the other jobs it ran with (but a
+ * TC_FP64 job whose residue images find no device memory runs on DMMA tiles).
  * ------------------------------------------------------------------------ */
 #define TC_JOB_DEVICE_INPUTS 1   /* tc_job arrays are DEVICE pointers, kept valid and
                                     unchanged by the caller until the job completes */
