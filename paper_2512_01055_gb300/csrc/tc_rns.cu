@@ -524,8 +524,8 @@ __global__ void rns_scales(int o, int v, Scales s) { finish_scales(o, v, s); }
 
 // All four steps by one CTA, for jobs where their launches take longer than
 // their work: up to SCALES_ONE rows of ovvv.
-// (Preparation, all steps in one launch against four: o=6 v=36 39 / 45 us, o=9 v=77
-// 153 / 160; where there are exponents 53 / 53 and 214 / 167, o=8 v=104 312 / 235.)
+// (Preparation, one launch against four: o=6 v=36 40 / 50 us, o=9 v=77 156 / 166,
+// o=8 v=104 218 / 230; where there are exponents 68 / 58, 258 / 173 and 428 / 241.)
 constexpr long long SCALES_ONE = 1 << 16;
 __global__ void __launch_bounds__(1024) rns_scales_one(int o, int v, Scales s) {
   wanted(o, v, s);
@@ -1435,7 +1435,9 @@ size_t rn_slot(int hps, int ncmax) { return (size_t)hps * (A_HALF + (size_t)ncma
 
 using RnKernel = void (*)(RnBatch);
 
-// The GEMM kernel instance for a widest N chunk of ncmax columns.
+// The GEMM kernel instance for a widest N chunk of ncmax columns: the columns of
+// the next instance are reduced along (W at o=6 v=64 379 us on <5>, 365 on a <4>;
+// v=96 1061 on <7>, 1037 on a <6>; eight instances compile in 11 s, five in 8).
 RnKernel rn_kernel(int ncmax) {
   const int u = ncmax / 16;
   return u <= 3 ? rns_gemm_kernel<3> : u <= 5 ? rns_gemm_kernel<5> : u <= 7 ? rns_gemm_kernel<7>
