@@ -53,14 +53,11 @@
 //
 // Weak triplets.  The grid is common to all triplets, so W of one whose
 // amplitudes or integrals are far below the others' keeps fewer bits, where FP64
-// accumulation keeps them relative to each product.  The energy kernel therefore
-// sums, beside E[4]_ST, what E[4]_ST would be if W had WEAK_RMS units of its
-// 64-bit fraction everywhere, and the DMMA kernel forms the triplets below that
 // accumulation keeps them relative to each product.  The rounding error of a
 // triplet's W follows from the norms of its rows.  The energy kernel sums, beside
 // E[4]_ST, what E[4]_ST would be if W were 2^49 times that error everywhere, and
 // the DMMA kernel forms the triplets below that again.
-
+#include <algorithm>
 #include <type_traits>
 
 #include "tc_internal.cuh"
